@@ -99,6 +99,7 @@ struct envar_handle_s {
     cudaEvent_t ev_solved0 = nullptr;   // member 0's pressure increment is final (group 0)
     cudaEvent_t ev_corr[ENVAR_MAX_GROUPS] = {};   // a group's correction has read member 0's increment
     int cimg_bytes = 0;
+    ClusterPlan *plan = nullptr, *plan_coarse = nullptr;   // cluster pressure solve / coarse V-cycle
     // reduced-space optimisers (allocated on first use)
     double *d_Y = nullptr, *d_h0 = nullptr, *d_smean = nullptr, *d_H = nullptr, *d_L = nullptr, *d_x = nullptr;
     int *d_info = nullptr;
@@ -383,8 +384,8 @@ static int build_geometry(envar_handle h)
         CK(cudaMemcpy(h->d_cimg, im.data(), im.size(), cudaMemcpyHostToDevice));
         h->cimg_bytes = lay.image_bytes;
     }
+    std::vector<uint8_t> op((size_t)S, 0);
     {   // level-0 open-face bits (W 1, E 2, S 4, N 8) of fluid cells
-        std::vector<uint8_t> op((size_t)S, 0);
         for (int j = 0; j < ny; ++j)
             for (int i = 0; i < nx; ++i) {
                 if (!F[(size_t)j * P + i]) continue;
@@ -403,6 +404,24 @@ static int build_geometry(envar_handle h)
         h->lev[0].cy = g.cy;
         h->lev[0].cxf = (float)g.cx;
         h->lev[0].cyf = (float)g.cy;
+    }
+    {   // the pressure solve, or the levels below the first, in a cluster per member
+        std::vector<ClusterHostLevel> cl(h->nlev);
+        for (int l = 0; l < h->nlev; ++l)
+            cl[l] = ClusterHostLevel{hl[l].nx, hl[l].ny, hl[l].P, hl[l].F.data(), l ? nullptr : op.data(), hl[l].cw.data(), hl[l].cs.data(),
+                                     h->lev[l].code != nullptr};
+        const ClusterAlloc al{[](void *owner, const void *src, size_t bytes) -> void * {
+                                  envar_handle o = (envar_handle)owner;
+                                  unsigned char *d = nullptr;
+                                  if (dalloc(o, &d, bytes)) return nullptr;
+                                  if (cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, o->st) != cudaSuccess) return nullptr;
+                                  return cudaStreamSynchronize(o->st) == cudaSuccess ? d : nullptr;
+                              },
+                              h, h->st};
+        if (coarse_bytes(h->ncoarse) <= (size_t)COARSE_SMEM_MAX) {
+            h->plan = cluster_plan(cl.data(), h->nlev, h->ncoarse, h->mixed, 0, al);
+            if (!h->plan && h->mixed) h->plan_coarse = cluster_plan(cl.data(), h->nlev, h->ncoarse, true, 1, al);
+        }
     }
     // coarse block must fit in shared memory
     if (coarse_bytes(h->ncoarse) > (size_t)COARSE_SMEM_MAX) {
@@ -934,6 +953,10 @@ extern "C" int envar_init(envar_handle *out, const envar_config *cfg, void *cuda
     }
     int rc = build_geometry(h);
     if (!rc) rc = alloc_buffers(h);
+    if (!rc && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // the buffers' clears, before work on h->st
+        set_err(h, "envar_init: %s", cudaGetErrorString(cudaGetLastError()));
+        rc = ENVAR_ECUDA;
+    }
     if (!rc) {
         PoissonCfg &pc = h->pc;
         pc.nlev = h->nlev; pc.ncoarse = h->ncoarse;
@@ -944,6 +967,8 @@ extern "C" int envar_init(envar_handle *out, const envar_config *cfg, void *cuda
         pc.rtol_abs = c.div_tol * h->g.hxy / h->g.dt;
         pc.cimg = h->d_cimg;
         pc.cimg_bytes = h->cimg_bytes;
+        pc.solve = h->plan;
+        pc.coarse = h->plan_coarse;
         {
             const Grid &g = h->g;
             auto split = [](double d, float *hi, float *lo) { *hi = (float)d; *lo = (float)(d - (double)*hi); };
@@ -983,6 +1008,8 @@ extern "C" int envar_destroy(envar_handle h)
     for (auto &row : h->adj_graph)
         for (auto &ge : row)
             if (ge) cudaGraphExecDestroy(ge);
+    cluster_plan_free(h->plan);
+    cluster_plan_free(h->plan_coarse);
     for (void *p : h->allocs) cudaFree(p);
     if (h->d_snap) cudaFree(h->d_snap);
     for (int k = 0; k < ENVAR_MAX_GROUPS; ++k) {

@@ -312,6 +312,26 @@ void launch_cost(const Grid &g, int M, const double *wf, const double *wd, const
 void launch_export_state(const Grid &g, const double *u, const double *v, const double *p, double *uo,
                          double *vo, double *po, cudaStream_t st);
 
+// Cluster pressure solve (k_cluster.cu): a member's whole solve, or the V-cycle of the levels below
+// the first, in one thread-block cluster.
+struct ClusterPlan;
+struct ClusterHostLevel {           // host copy of a multigrid level, pitch P
+    int nx, ny, P;
+    const uint8_t *F, *open;        // fluid cells; open-face bits (first level)
+    const double *cw, *cs;          // west / south face conductances
+    bool coded;                     // the tiled smoother holds this level's conductances as codes
+};
+struct ClusterAlloc {               // device copy of a host array, owned by the handle (nullptr: out of memory)
+    void *(*copy)(void *owner, const void *h, size_t bytes);
+    void *owner;
+    cudaStream_t st;
+    void *operator()(const void *h, size_t bytes) const { return copy(owner, h, bytes); }
+};
+// The plan for a grid (la 0: the whole solve; la 1: the V-cycle from level 1 on), nullptr where it does
+// not fit a cluster.
+ClusterPlan *cluster_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, bool mixed, int la, const ClusterAlloc &alloc);
+void cluster_plan_free(ClusterPlan *p);
+
 // Poisson kernels (k_poisson.cu).  TM = multigrid / inner-CG precision.
 struct PoissonBufs {
     MixState ms;                    // mixed mode: df64 b and x live here
@@ -335,6 +355,8 @@ struct PoissonCfg {
     MixConst mc;
     const unsigned char *cimg;      // coarse-block shared-memory image of the coarse levels' constants
     int cimg_bytes;                 // its size (a multiple of 16)
+    ClusterPlan *solve;             // the whole solve in a cluster per member, or
+    ClusterPlan *coarse;            // the V-cycle's levels from 1 on (FP32); nullptr: tiled kernels
 };
 // Shared-memory layout of the coarse block (levels lc .. nlev-1).  The constant part (per level:
 // west-face conductances [ny][nx+1], south-face conductances [ny+1][nx] in TM, fluid flags
@@ -364,6 +386,11 @@ int launch_poisson_single(int which, const Grid &g, const Level *lev, int M, con
 template <class TM>
 void launch_pressure_solve(const Grid &g, const Level *lev, int M, const PoissonBufs &B, const PoissonCfg &pc,
                            const Partials &pt, MemberCtl *ctl, cudaStream_t st);
+
+template <class TM>
+void launch_cluster_solve(const Grid &g, const Level &L0, int M, const PoissonBufs &B, const PoissonCfg &pc, const Partials &pt,
+                          MemberCtl *ctl, cudaStream_t st);
+void launch_cluster_vcycle(int M, const float *f, float *e, const PoissonCfg &pc, MemberCtl *ctl, int inner_guard, cudaStream_t st);
 
 // Mixed-precision kernels (k_mixed.cu)
 void launch_load_ic_mx(const Grid &g, const double *u0, const double *v0, const MixState &s0, cudaStream_t st);

@@ -1133,7 +1133,9 @@ static void vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B,
     // level 0 input f = r (inner residual), output z
     const T *f0 = (const T *)B.r;
     T *z = (T *)B.z;
-    const int lc = pc.ncoarse;
+    // levels from 1 on in a cluster per member where a plan exists (float only)
+    const bool cl = pc.coarse != nullptr && sizeof(T) == 4;
+    const int lc = cl ? 1 : pc.ncoarse;
     // descend
     for (int l = 0; l < lc; ++l) {
         const Level &L = lev[l];
@@ -1146,7 +1148,9 @@ static void vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B,
                          ctl, inner_guard);
     }
     // coarse block
-    {
+    if (cl) {
+        launch_cluster_vcycle(M, (const float *)B.lev_f[1], (float *)B.lev_e[1], pc, ctl, inner_guard, st);
+    } else {
         CoarseArgs ca;
         const size_t smem = coarse_args<T>(lev, pc, inner_guard, &ca);
         const T *fin = (lc == 0) ? f0 : (const T *)B.lev_f[lc];
@@ -1287,6 +1291,10 @@ void launch_pressure_solve(const Grid &g, const Level *lev, int M, const Poisson
 {
     RedCtx rc = make_ctx(pt);
     const Level &L0 = lev[0];
+    if (pc.solve) {
+        launch_cluster_solve<TM>(g, L0, M, B, pc, pt, ctl, st);
+        return;
+    }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaGraph_t graph = nullptr;
     const cudaGraphNode_t *deps = nullptr;
