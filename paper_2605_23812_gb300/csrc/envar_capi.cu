@@ -1613,9 +1613,7 @@ extern "C" int envar_h1_smooth(envar_handle h, const double *g_dev, double *gs_d
     if (!h || !g_dev || !gs_dev || !(l_sob >= 0.0)) return ENVAR_EINVAL;
     const int n = h->ncc;
     if (!h->d_h1) { DA(h->d_h1, 3 * (size_t)n); DA(h->d_h1it, 2); }
-    for (int comp = 0; comp < 2; ++comp)
-        launch_h1_cg(n, h->d_cnb, h->g.dx, h->g.dy, l_sob, g_dev + (size_t)comp * n, gs_dev + (size_t)comp * n, h->d_h1,
-                     1e-13, 4 * n + 100, h->d_h1it + comp, h->st);
+    launch_h1_cg(n, h->nrx, h->d_cnb, h->g.dx, h->g.dy, l_sob, g_dev, gs_dev, h->d_h1, 1e-13, 4 * n + 100, h->d_h1it, h->st);
     int it[2] = {0, 0};
     CK(cudaMemcpyAsync(it, h->d_h1it, sizeof(int) * 2, cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));

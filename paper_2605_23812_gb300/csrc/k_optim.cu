@@ -326,13 +326,189 @@ __global__ void __launch_bounds__(1024) k_h1_cg(int n, const int *__restrict__ n
     if (tid == 0) *iters = done ? it : -it;
 }
 
-void launch_h1_cg(int n, const int *nb, double dx, double dy, double l_sob, const double *g, double *x, double *work,
+// The same iteration with each component on one thread-block cluster: rank k of C holds the cells
+// [k len, (k + 1) len) in shared memory with p on a halo of hx cells to either side (hx: the widest row of
+// the control rectangle, so every neighbour of an own cell lies within).  Two cluster barriers per
+// iteration, one behind each inner product: p of the halo is not sent but advanced in place from the
+// neighbour rank's r, which the second barrier has made final.  Each warp pushes its partial to every
+// rank and one warp adds them in rank order, so all ranks hold the same scalars and leave together.
+//
+// 512 x 256 (11454 cells, 16 blocks of 716): 12.55 ms -> 0.78 ms for both components, one block each before.
+// FP64 issue (1.67 multiply-adds per clock and SM, measured) and the two exchanges bound it about equally, so eight
+// warps of a few cells each beat one cell per thread: the reductions cost per warp.  Missing neighbours read a
+// zero slot and the diagonal is kept, five operations per cell instead of eight with branches.
+static constexpr int H1_THREADS = 256, H1_MAXC = 16;
+
+__device__ __forceinline__ unsigned int h1_remote(const void *p, int rank)
+{
+    unsigned int r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned int)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void h1_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The block's values of v to slot[rank * warps + warp] of every rank; after the barrier, warp 0 returns the
+// sum over the cluster (the other warps' result is not used).
+__device__ __forceinline__ double h1_cluster_sum(double v, double *slot, int C, int rank)
+{
+    constexpr int W = H1_THREADS / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    v = warp_sum(v);
+    if (lane < C)
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(h1_remote(slot + rank * W + warp, lane)), "d"(v) : "memory");
+    h1_cluster_sync();
+    double s = 0.0;
+    if (warp == 0) {
+        for (int q = lane; q < C * W; q += 32) s += slot[q];
+        s = warp_sum(s);
+    }
+    return s;
+}
+
+static size_t h1_smem(int len, int hx)
+{
+    return sizeof(double) * (2 * H1_MAXC * (H1_THREADS / 32) + 4 + 4 * (size_t)len + (size_t)len + 2 * (size_t)hx + 1) +
+           sizeof(int) * 4 * (size_t)len;
+}
+
+__global__ void __launch_bounds__(H1_THREADS) k_h1_cluster(int n, int C, int len, int hx, const int *__restrict__ nb, double cxl,
+                                                           double cyl, double scale, const double *g, double *x_out,
+                                                           double rtol, int max_it, int *iters)
+{
+    extern __shared__ double sh[];
+    constexpr int W = H1_THREADS / 32, NT = H1_THREADS;
+    double *slots = sh, *sc = slots + 2 * H1_MAXC * W, *r = sc + 4, *x = r + len, *ap = x + len, *dg = ap + len, *p = dg + len;
+    int *nbl = reinterpret_cast<int *>(p + len + 2 * hx + 1);
+    const int t = threadIdx.x, comp = blockIdx.x / C, rank = blockIdx.x % C;
+    const int a0 = min(rank * len, n), own = min(len, n - a0);
+    const int lo = max(0, a0 - hx), hi = min(n, a0 + own + hx);
+    const int p0 = a0 - lo + 1;                              // slot of own cell 0 in p; slot 0 is zero
+    g += (long long)comp * n;
+    x_out += (long long)comp * n;
+    for (int q = t; q < hi - lo; q += NT) p[q + 1] = scale * g[lo + q];
+    if (t == 0) p[0] = 0.0;
+    double acc = 0.0;
+    for (int q = t; q < own; q += NT) {
+        const double b = scale * g[a0 + q];
+        double d = 1.0;
+        for (int k = 0; k < 4; ++k) {
+            const int c = nb[k * n + a0 + q];
+            nbl[k * len + q] = (c >= lo && c < hi) ? c - lo + 1 : 0;
+            if (c >= 0) d += (k < 2) ? cxl : cyl;
+        }
+        dg[q] = d;
+        r[q] = b;
+        x[q] = 0.0;
+        acc += b * b;
+    }
+    h1_cluster_sync();                                       // every rank runs before the first remote store
+    const double bb = h1_cluster_sum(acc, slots, C, rank);
+    if (t == 0) { sc[0] = bb; sc[1] = 0.0; sc[2] = (bb > 0.0) ? 0.0 : 1.0; sc[3] = bb; }
+    __syncthreads();
+    int it = 0;
+    bool done = sc[2] != 0.0;
+    const int nhalo = (hi - lo) - own, before = a0 - lo;
+    while (!done && it < max_it) {
+        acc = 0.0;
+#pragma unroll 2
+        for (int q = t; q < own; q += NT) {
+            const double pq = p[p0 + q];
+            const double sx = p[nbl[q]] + p[nbl[len + q]], sy = p[nbl[2 * len + q]] + p[nbl[3 * len + q]];
+            const double a = fma(-cyl, sy, fma(-cxl, sx, dg[q] * pq));
+            ap[q] = a;
+            acc = fma(pq, a, acc);
+        }
+        const double pAp = h1_cluster_sum(acc, slots + H1_MAXC * W, C, rank);
+        if (t == 0) sc[1] = sc[0] / pAp;
+        __syncthreads();
+        const double alpha = sc[1];
+        acc = 0.0;
+#pragma unroll 2
+        for (int q = t; q < own; q += NT) {
+            x[q] = fma(alpha, p[p0 + q], x[q]);
+            const double rq = fma(-alpha, ap[q], r[q]);
+            r[q] = rq;
+            acc = fma(rq, rq, acc);
+        }
+        const double rr1 = h1_cluster_sum(acc, slots, C, rank);
+        if (t == 0) {
+            sc[1] = rr1 / sc[0];
+            sc[0] = rr1;
+            sc[2] = (rr1 <= rtol * rtol * sc[3]) ? 1.0 : 0.0;
+        }
+        // the neighbour ranks' r for the halo, in flight behind the scalars
+        double hr[2] = {0.0, 0.0};
+        auto halo_r = [&](int h) {
+            const int c = h < before ? lo + h : a0 + own + (h - before), k = c / len;
+            double v;
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(h1_remote(r + (c - k * len), k)) : "memory");
+            return v;
+        };
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (t + u * NT < nhalo) hr[u] = halo_r(t + u * NT);
+        __syncthreads();
+        ++it;
+        done = sc[2] != 0.0;
+        const double beta = sc[1];
+        if (done) break;
+        for (int h = t, u = 0; h < nhalo; h += NT, ++u) {
+            double &ph = p[1 + (h < before ? h : own + h)];
+            ph = fma(beta, ph, u == 0 ? hr[0] : u == 1 ? hr[1] : halo_r(h));
+        }
+        for (int q = t; q < own; q += NT) p[p0 + q] = fma(beta, p[p0 + q], r[q]);
+        __syncthreads();
+    }
+    for (int q = t; q < own; q += NT) x_out[a0 + q] = x[q];
+    if (rank == 0 && t == 0) iters[comp] = done ? it : -it;
+    h1_cluster_sync();                                       // no rank leaves while others may read its r
+}
+
+// Both components: on clusters of up to 16 blocks where their shared memory holds the control cells (70 000 at rows of
+// 200; 57 bytes per cell), else one after the other in one block.
+void launch_h1_cg(int n, int row, const int *nb, double dx, double dy, double l_sob, const double *g, double *x, double *work,
                   double rtol, int max_it, int *iters, cudaStream_t st)
 {
-    const double l2 = l_sob * l_sob;
-    k_h1_cg<<<1, 1024, 0, st>>>(n, nb, l2 / (dx * dx), l2 / (dy * dy), 1.0 + l2, g, x, work, work + n, work + 2 * n,
-                               rtol, max_it, iters);
-    count_launches(1);
+    const double l2 = l_sob * l_sob, cxl = l2 / (dx * dx), cyl = l2 / (dy * dy);
+    // 256 cells per block fill its eight warps once; 16 blocks is the largest cluster
+    for (int C = std::min(H1_MAXC, std::max(1, cdiv(n, H1_THREADS))); C >= 1; C = C > 8 ? 8 : 0) {
+        const int len = cdiv(n, C);
+        const size_t smem = h1_smem(len, row);
+        if (smem > 220 * 1024) continue;
+        if (cudaFuncSetAttribute(k_h1_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(k_h1_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(2 * C);
+        lc.blockDim = dim3(H1_THREADS);
+        lc.dynamicSmemBytes = smem;
+        lc.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_h1_cluster, &lc) != cudaSuccess || fit < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        if (cudaLaunchKernelEx(&lc, k_h1_cluster, n, C, len, row, nb, cxl, cyl, 1.0 + l2, g, x, rtol, max_it, iters) == cudaSuccess) {
+            count_launches(1);
+            return;
+        }
+        cudaGetLastError();
+    }
+    for (int comp = 0; comp < 2; ++comp)
+        k_h1_cg<<<1, 1024, 0, st>>>(n, nb, cxl, cyl, 1.0 + l2, g + (size_t)comp * n, x + (size_t)comp * n, work, work + n,
+                                    work + 2 * (size_t)n, rtol, max_it, iters + comp);
+    count_launches(2);
 }
 
 // y = a x (elementwise scale), and the directional derivative d = g^T p of two n-vectors.
