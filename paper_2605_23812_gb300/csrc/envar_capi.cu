@@ -257,6 +257,24 @@ static int build_geometry(envar_handle h)
     CK(cudaMemcpy(duin, uin.data(), sizeof(double) * ny, cudaMemcpyHostToDevice));
     g.fluid = dF; g.uk = duk; g.vk = dvk; g.u_in = duin;
     {
+        std::vector<unsigned int> tiles;
+        for (int tj = 0; tj * 8 <= ny; ++tj)
+            for (int ti = 0; ti * 32 <= nx; ++ti) {
+                bool any = false;
+                for (int j = tj * 8; j < std::min(tj * 8 + 8, ny + 1); ++j)
+                    for (int i = ti * 32; i < std::min(ti * 32 + 32, nx + 1); ++i) {
+                        const uint8_t a = uk[(size_t)j * P + i], b = vk[(size_t)j * P + i];
+                        any = any || F[(size_t)j * P + i] || a == FK_UNK || a == FK_INLET || a == FK_OUTLET || b == FK_UNK;
+                    }
+                if (any) tiles.push_back((unsigned int)ti | ((unsigned int)tj << 16));
+            }
+        unsigned int *dt;
+        DA(dt, tiles.size());
+        CK(cudaMemcpy(dt, tiles.data(), sizeof(unsigned int) * tiles.size(), cudaMemcpyHostToDevice));
+        g.tiles = dt;
+        g.ntiles = (int)tiles.size();
+    }
+    {
         std::vector<float> ih((size_t)ny), il((size_t)ny);
         for (int j = 0; j < ny; ++j) {
             ih[j] = (float)uin[j];
@@ -533,6 +551,7 @@ static int alloc_buffers(envar_handle h)
         DA(ms.p, n0); DA(ms.Ru, 2 * n0); DA(ms.Rv, 2 * n0);
         ms.rstride = (long long)n0;
         DA(ms.bh, n0); DA(ms.bl, n0); DA(ms.xh, n0); DA(ms.xl, n0);
+        for (float *q : {ms.ush, ms.usl, ms.vsh, ms.vsl, ms.bh, ms.bl}) CK(cudaMemset(q, 0, sizeof(float) * n0));
         if (h->cfg.guess_extrapolation) DA(ms.xp, n0);
         if (h->cfg.cost_mode == ENVAR_COST_DOMAIN) DA(ms.wf, 6 * n0);
         if (h->cfg.cost_mode == ENVAR_COST_DOMAIN && h->N > 0) DA(ms.wd, 4 * n0);
@@ -545,6 +564,7 @@ static int alloc_buffers(envar_handle h)
         DA(h->d_u0, S); DA(h->d_v0, S);
         DA(h->d_u, n0); DA(h->d_v, n0); DA(h->d_us, n0); DA(h->d_vs, n0); DA(h->d_p, n0);
         DA(h->pb.x, n0); DA(h->pb.b, n0);
+        for (double *q : {h->d_us, h->d_vs, h->pb.b}) CK(cudaMemset(q, 0, sizeof(double) * n0));
         h->tend_bytes = tsz * n0;
         char *a, *b;
         DA(a, h->tend_bytes); DA(b, h->tend_bytes);

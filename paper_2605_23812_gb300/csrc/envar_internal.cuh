@@ -57,6 +57,10 @@ struct Grid {
     int ia, ja, nrx, nry;   // control rectangle (cells)
     int n_steps, n_window;
     double conv_speed;
+    // the 32 x 8 tiles (column | row << 16) that hold a fluid cell or a face that is not a wall: the
+    // flow kernels visit these alone, walls and solid keep the zeros they start with
+    const unsigned int *tiles;
+    int ntiles;
 };
 
 // Per-member control block in device memory.

@@ -144,9 +144,8 @@ __global__ void __launch_bounds__(256) k_predict(Grid g, const double *__restric
                                                  double *__restrict__ vs, const double *__restrict__ ubc,
                                                  const double *__restrict__ frect, const MemberCtl *__restrict__ ctl)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    int m = blockIdx.z;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x, j = (tile >> 16) * 8 + threadIdx.y, m = blockIdx.y;
     if (i > g.nx || j > g.ny) return;
     const long long off = (long long)m * g.S;
     const double *um = u + off, *vm = v + off, *pm = p + off;
@@ -211,7 +210,7 @@ void launch_predict(const Grid &g, int M, const double *u, const double *v, cons
                     double *us, double *vs, const double *ubc, const double *frect, const MemberCtl *ctl,
                     cudaStream_t st)
 {
-    dim3 blk(32, 8), grd(cdiv(g.nx + 1, 32), cdiv(g.ny + 1, 8), M);
+    dim3 blk(32, 8), grd(g.ntiles, M);
     k_predict<TR><<<grd, blk, 0, st>>>(g, u, v, p, Ru, Rv, us, vs, ubc, frect, ctl);
     count_launches(1);
 }
@@ -225,9 +224,8 @@ template void launch_predict<double>(const Grid &, int, const double *, const do
 // ---------------------------------------------------------------------------- rhs
 __global__ void k_rhs(Grid g, const double *__restrict__ us, const double *__restrict__ vs, double *__restrict__ b)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    int m = blockIdx.z;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x, j = (tile >> 16) * 8 + threadIdx.y, m = blockIdx.y;
     if (i >= g.nx || j >= g.ny) return;
     const long long off = (long long)m * g.S, c = (long long)j * g.P + i;
     double r = 0.0;
@@ -241,7 +239,7 @@ __global__ void k_rhs(Grid g, const double *__restrict__ us, const double *__res
 
 void launch_rhs(const Grid &g, int M, const double *us, const double *vs, double *b, MemberCtl *, cudaStream_t st)
 {
-    dim3 blk(32, 8), grd(cdiv(g.nx, 32), cdiv(g.ny, 8), M);
+    dim3 blk(32, 8), grd(g.ntiles, M);
     k_rhs<<<grd, blk, 0, st>>>(g, us, vs, b);
     count_launches(1);
 }
@@ -313,9 +311,8 @@ __global__ void __launch_bounds__(256) k_correct(Grid g, double x0, double y0, d
                                                  double *__restrict__ series, Partials pt, MemberCtl *ctl,
                                                  double div_tol, long long nfluid)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int j = blockIdx.y * blockDim.y + threadIdx.y;
-    int m = blockIdx.z;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x, j = (tile >> 16) * 8 + threadIdx.y, m = blockIdx.y;
     const long long off = (long long)m * g.S;
     const long long c = (long long)j * g.P + i;
     const double *usm = us + off, *vsm = vs + off, *xm = x + off;
@@ -373,7 +370,7 @@ __global__ void __launch_bounds__(256) k_correct(Grid g, double x0, double y0, d
     }
     bad = __syncthreads_or(bad);
     if (tid == 0 && bad) atomicOr(&ctl[m].status, bad);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+    if (blockIdx.x == 0 && tid == 0) {
         double dv = g.dt * pt.red[m].val[RS_RMAX] / g.hxy;
         if (dv > ctl[m].max_div) ctl[m].max_div = dv;
         if (!(dv <= div_tol)) ctl[m].status |= ENVAR_ST_DIVERGENCE;
@@ -391,7 +388,7 @@ void launch_correct(const Grid &g, double x0, double y0, int M, double *u, doubl
                     int want_welford, double *series, const Partials &pt, MemberCtl *ctl, double div_tol,
                     long long nfluid, cudaStream_t st)
 {
-    dim3 blk(32, 8), grd(cdiv(g.nx + 1, 32), cdiv(g.ny + 1, 8), M);
+    dim3 blk(32, 8), grd(g.ntiles, M);
     k_correct<<<grd, blk, 0, st>>>(g, x0, y0, u, v, p, us, vs, x, wf, wd, ref, want_welford, series, pt, ctl,
                                    div_tol, nfluid);
     count_launches(1);
@@ -402,8 +399,8 @@ void launch_correct(const Grid &g, double x0, double y0, int M, double *u, doubl
 // scales with |x|), so the guess is re-centred on the fluid mean once the step has used it.
 __global__ void k_recenter(Grid g, double *__restrict__ x, Partials pt, long long nfluid)
 {
-    const int m = blockIdx.z;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x, j = (tile >> 16) * 8 + threadIdx.y, m = blockIdx.y;
     if (i >= g.nx || j >= g.ny) return;
     const long long c = (long long)j * g.P + i;
     if (g.fluid[c]) x[(long long)m * g.S + c] -= pt.red[m].val[RS_XSUM] / (double)nfluid;
@@ -411,7 +408,7 @@ __global__ void k_recenter(Grid g, double *__restrict__ x, Partials pt, long lon
 
 void launch_recenter(const Grid &g, int M, double *x, const Partials &pt, long long nfluid, cudaStream_t st)
 {
-    dim3 blk(32, 8), grd(cdiv(g.nx, 32), cdiv(g.ny, 8), M);
+    dim3 blk(32, 8), grd(g.ntiles, M);
     k_recenter<<<grd, blk, 0, st>>>(g, x, pt, nfluid);
     count_launches(1);
 }

@@ -252,9 +252,10 @@ __global__ void __launch_bounds__(PR_TX *PR_TY, 6) k_predict_rhs_mx(Grid g, MixC
     __shared__ float svh[PR_TY + 1][PR_TX], svl[PR_TY + 1][PR_TX];
     __shared__ float s_xmean;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i0 = blockIdx.x * PR_TX, j0 = blockIdx.y * PR_TY;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i0 = (tile & 0xffffu) * PR_TX, j0 = (tile >> 16) * PR_TY;
     const int i = i0 + tx, j = j0 + ty;
-    const int m = blockIdx.z;
+    const int m = blockIdx.y;
     const long long off = (long long)m * g.S;
     const int step = ctl[m].step;
     const bool first = (step == 1);
@@ -319,7 +320,7 @@ void launch_predict_rhs_mx(const Grid &g, const MixConst &K, int M, const MixSta
                            const float *inh, const float *inl, const MemberCtl *ctl, const MemberRed *red,
                            long long nfluid, cudaStream_t st)
 {
-    dim3 blk(PR_TX, PR_TY), grd(cdiv(g.nx + 1, PR_TX), cdiv(g.ny + 1, PR_TY), M);
+    dim3 blk(PR_TX, PR_TY), grd(g.ntiles, M);
     k_predict_rhs_mx<<<grd, blk, 0, st>>>(g, K, s, ubc, inh, inl, ctl, red, (float)(1.0 / (double)nfluid));
     count_launches(1);
 }
@@ -609,9 +610,10 @@ __global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixSt
                                                     int want_welford, double *__restrict__ series, Partials pt,
                                                     MemberCtl *ctl, double div_tol, long long nfluid)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int m = blockIdx.z;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x;
+    const int j = (tile >> 16) * 8 + threadIdx.y;
+    const int m = blockIdx.y;
     const long long off = (long long)m * g.S;
     const int P = g.P;
     const float *__restrict__ ush = s.ush + off;
@@ -684,7 +686,7 @@ __global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixSt
     }
     bad = __syncthreads_or(bad);
     if (tid == 0 && bad) atomicOr(&ctl[m].status, bad);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+    if (blockIdx.x == 0 && tid == 0) {
         double dv = g.dt * pt.red[m].val[RS_RMAX] / g.hxy;
         if (dv > ctl[m].max_div) ctl[m].max_div = dv;
         if (!(dv <= div_tol)) ctl[m].status |= ENVAR_ST_DIVERGENCE;
@@ -701,7 +703,7 @@ void launch_correct_mx(const Grid &g, const MixConst &K, int M, const MixState &
                        double y0, int want_welford, double *series, const Partials &pt, MemberCtl *ctl,
                        double div_tol, long long nfluid, cudaStream_t st)
 {
-    dim3 blk(32, 8), grd(cdiv(g.nx + 1, 32), cdiv(g.ny + 1, 8), M);
+    dim3 blk(32, 8), grd(g.ntiles, M);
     k_correct_mx<<<grd, blk, 0, st>>>(g, K, s, ref, x0, y0, want_welford, series, pt, ctl, div_tol, nfluid);
     count_launches(1);
 }
