@@ -260,12 +260,12 @@ static int build_geometry(envar_handle h)
         std::vector<unsigned int> tiles;
         for (int tj = 0; tj * 8 <= ny; ++tj)
             for (int ti = 0; ti * 32 <= nx; ++ti) {
+                const int i0 = ti * 32, w = std::min(32, nx + 1 - i0);
                 bool any = false;
-                for (int j = tj * 8; j < std::min(tj * 8 + 8, ny + 1); ++j)
-                    for (int i = ti * 32; i < std::min(ti * 32 + 32, nx + 1); ++i) {
-                        const uint8_t a = uk[(size_t)j * P + i], b = vk[(size_t)j * P + i];
-                        any = any || F[(size_t)j * P + i] || a == FK_UNK || a == FK_INLET || a == FK_OUTLET || b == FK_UNK;
-                    }
+                for (int j = tj * 8; j < std::min(tj * 8 + 8, ny + 1) && !any; ++j) {
+                    auto has = [&](const std::vector<uint8_t> &k, int v) { return std::memchr(&k[(size_t)j * P + i0], v, w) != nullptr; };
+                    any = has(F, 1) || has(uk, FK_UNK) || has(uk, FK_INLET) || has(uk, FK_OUTLET) || has(vk, FK_UNK);
+                }
                 if (any) tiles.push_back((unsigned int)ti | ((unsigned int)tj << 16));
             }
         unsigned int *dt;
@@ -273,6 +273,16 @@ static int build_geometry(envar_handle h)
         CK(cudaMemcpy(dt, tiles.data(), sizeof(unsigned int) * tiles.size(), cudaMemcpyHostToDevice));
         g.tiles = dt;
         g.ntiles = (int)tiles.size();
+        std::vector<uint8_t> strips((size_t)cdiv(nx, 64) * cdiv(ny, 4), 0);
+        for (int j = 0; j < ny; ++j)
+            for (int k = 0; k < cdiv(nx, 64); ++k) {
+                uint8_t &q = strips[(size_t)(j / 4) * cdiv(nx, 64) + k];
+                q = q || std::memchr(&F[(size_t)j * P + k * 64], 1, std::min(64, nx - k * 64)) != nullptr;
+            }
+        uint8_t *ds;
+        DA(ds, strips.size());
+        CK(cudaMemcpy(ds, strips.data(), strips.size(), cudaMemcpyHostToDevice));
+        g.strips = ds;
     }
     {
         std::vector<float> ih((size_t)ny), il((size_t)ny);
@@ -418,6 +428,13 @@ static int build_geometry(envar_handle h)
         DA(dop, S);
         CK(cudaMemcpy(dop, op.data(), S, cudaMemcpyHostToDevice));
         h->lev[0].open = dop;
+        for (int k = 0; k < 3; ++k) {
+            const std::vector<uint8_t> t = smooth_tiles(nx, ny, P, F.data(), h->mixed, k + 1);
+            uint8_t *dt;
+            DA(dt, t.size());
+            CK(cudaMemcpy(dt, t.data(), t.size(), cudaMemcpyHostToDevice));
+            h->lev[0].tile_fluid[k] = dt;
+        }
         h->lev[0].cx = g.cx;
         h->lev[0].cy = g.cy;
         h->lev[0].cxf = (float)g.cx;
@@ -584,15 +601,19 @@ static int alloc_buffers(envar_handle h)
     {
         char *r, *e, *z, *q, *pv;
         DA(r, tsz * n0); DA(e, tsz * n0); DA(z, tsz * n0); DA(q, tsz * n0); DA(pv, 2 * tsz * n0);
+        // the kernels skip regions without a fluid cell and rely on zeros there
+        for (char *a : {r, e, z, q, pv, pv + tsz * n0}) CK(cudaMemset(a, 0, tsz * n0));
         h->pb.r = r; h->pb.e = e; h->pb.z = z; h->pb.q = q; h->pb.pv = pv; h->pb.pv1 = pv + tsz * n0;
         for (int l = 1; l < h->nlev; ++l) {
             char *le, *lf;
             DA(le, tsz * (size_t)h->lev[l].S * M); DA(lf, tsz * (size_t)h->lev[l].S * M);
+            if (l == 1) CK(cudaMemset(lf, 0, tsz * (size_t)h->lev[l].S * M));
             h->pb.lev_e[l] = le; h->pb.lev_f[l] = lf;
         }
         for (int l = 0; l < h->ncoarse; ++l) {
             char *lt;
             DA(lt, tsz * (size_t)h->lev[l].S * M);
+            if (l == 0) CK(cudaMemset(lt, 0, tsz * (size_t)h->lev[l].S * M));
             h->pb.lev_t[l] = lt;
         }
     }
@@ -1919,6 +1940,9 @@ extern "C" int envar_apply_preconditioner(envar_handle h, const double *r_dev, d
         launch_vcycle<double>(h->g, h->lev, h->Mall, h->pb, h->pc, h->pt, h->d_ctl, h->st);
         launch_cells_out<double>(h->g, (const double *)h->pb.z, z_dev, h->st);
     }
+    // r_dev may be nonzero in solid cells: the solves count on zeros there
+    CK(cudaMemsetAsync(h->pb.r, 0, tsz * (size_t)h->g.S * h->Mall, h->st));
+    CK(cudaMemsetAsync(h->pb.lev_f[1], 0, tsz * (size_t)h->lev[1].S * h->Mall, h->st));
     CK(cudaStreamSynchronize(h->st));
     CK(cudaGetLastError());
     return ENVAR_OK;

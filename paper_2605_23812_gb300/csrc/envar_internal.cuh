@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace envar {
 
 // FK_SOLID faces take the odd mirror of their fluid-side neighbour inside stencils (no slip),
@@ -42,6 +44,8 @@ struct Level {
     const uint16_t *code;
     const float *ktabf;
     const double *ktabd;
+    // level 0 only: for 1, 2, 3 sweep pairs, whether each tile of the warp-row smoother holds a fluid cell
+    const uint8_t *tile_fluid[3];
 };
 
 struct Grid {
@@ -61,6 +65,8 @@ struct Grid {
     // flow kernels visit these alone, walls and solid keep the zeros they start with
     const unsigned int *tiles;
     int ntiles;
+    // per 64 x 4 strip of cells, row by row of strips: whether it holds a fluid cell
+    const uint8_t *strips;
 };
 
 // Per-member control block in device memory.
@@ -373,6 +379,7 @@ struct CoarseLayout {
 CoarseLayout coarse_layout(const Level *lev, int lc, int nlev, size_t tsz);
 template <class TM> void prepare_poisson_kernels();
 // The largest number of r^T z partials (blocks per member) a level-0 post-smoothing launch leaves (any sweep count).
+std::vector<uint8_t> smooth_tiles(int nx, int ny, int P, const uint8_t *fluid, bool mixed, int pairs);
 int rz_parts_max(const Level &L0, bool mixed);
 template <class TM>
 void launch_vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B, const PoissonCfg &pc,

@@ -350,8 +350,10 @@ __global__ void __launch_bounds__(OR_WARPS * 32) k_outer_residual_mx(Grid g, Lev
     const long long off = (long long)m * g.S;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int iL = blockIdx.x * 64 + 2 * lane;
-    const bool colok = iL < g.nx;                               // nx is even: both cells of the pair
     const int j0 = (blockIdx.y * OR_WARPS + w) * OR_ROWS;
+    // a strip without a fluid cell: r and e stay zero, nothing to add to the partials
+    const bool strip = j0 < g.ny && g.strips[(j0 / OR_ROWS) * gridDim.x + blockIdx.x];
+    const bool colok = strip && iL < g.nx;                      // nx is even: both cells of the pair
     const float *xhm = xh + off, *xlm = xl + off;
     float2 xrh[NR], xrl[NR], brh[R], brl[R];
     f2 xw[R], xe[R];
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(OR_WARPS * 32) k_outer_residual_mx(Grid g, Lev
         brh[q] = brl[q] = make_float2(0.f, 0.f);
         xw[q] = xe[q] = f2{0.f, 0.f};
         ob[q] = fl[q] = 0u;
-        if (j < g.ny) {
+        if (strip && j < g.ny) {
             const long long c = (long long)j * g.P + iL;
             if (colok) {
                 brh[q] = ld_early_nc(reinterpret_cast<const float2 *>(bh + off + c));
@@ -397,7 +399,7 @@ __global__ void __launch_bounds__(OR_WARPS * 32) k_outer_residual_mx(Grid g, Lev
     };
     float rmax = 0.f;
     f2 xs{0.f, 0.f};
-    if (j0 < g.ny) {
+    if (strip) {
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             const int j = j0 + q;
@@ -458,10 +460,11 @@ __global__ void __launch_bounds__(128) k_axpy_last_mx(Grid g, float *__restrict_
     // the data first (none of it depends on the control word or on alpha); pairs past nx are not
     // touched (nx is even: pairs are whole)
     float2 ev[2], pv[2], x0[2], x1[2];
+    const bool strip = i < g.nx && g.strips[(j >> 2) * ((g.nx + 63) >> 6) + (i >> 6)];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         ev[h] = pv[h] = x0[h] = x1[h] = make_float2(0.f, 0.f);
-        if (i + 2 * h < g.nx) {
+        if (strip && i + 2 * h < g.nx) {
             ev[h] = ld_early_nc(reinterpret_cast<const float2 *>(e + c + 2 * h));
             pv[h] = ld_early_nc(reinterpret_cast<const float2 *>(p + c + 2 * h));
             x0[h] = ld_early(reinterpret_cast<const float2 *>(xh + c + 2 * h));

@@ -18,6 +18,7 @@
 // publishes the scalar and the convergence flags in the member's control block.  Every loop is a
 // fixed number of launches (graph friendly); converged members' blocks exit at once.
 #include <algorithm>
+#include <cstring>
 
 #include "df64.cuh"
 #include "envar_internal.cuh"
@@ -243,8 +244,10 @@ __global__ void __launch_bounds__(SPMV_WARPS * 32) k_spmv0(Grid g, Level L0, con
     const long long off = (long long)m * g.S;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int iL = blockIdx.x * 64 + 2 * lane;
-    const bool colok = iL + 1 < g.nx;                       // nx is even
     const int j0 = (blockIdx.y * SPMV_WARPS + w) * SPMV_ROWS;
+    // a strip without a fluid cell stays zero (z, p and q are zero there) and adds nothing to p^T q
+    const bool strip = j0 < g.ny && g.strips[(j0 / SPMV_ROWS) * gridDim.x + blockIdx.x];
+    const bool colok = strip && iL + 1 < g.nx;              // nx is even
     const T *zm = z + off, *pm = pold + off;
     // every load of the warp's rows first (rows j0 - 1 .. j0 + R; z, and p for k > 0; the strip's
     // edge cells; the open-face bits): none depends on the control word or on beta
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(SPMV_WARPS * 32) k_spmv0(Grid g, Level L0, con
         const int j = j0 + r;
         zw[r] = ze[r] = pw[r] = pe[r] = (T)0;
         ob[r] = 0u;
-        if (j < g.ny) {
+        if (strip && j < g.ny) {
             const long long c = (long long)j * g.P + iL;
             if (colok) ob[r] = ld_early_nc_u16(L0.open + c);
             if (lane == 0 && iL >= 1) {
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(SPMV_WARPS * 32) k_spmv0(Grid g, Level L0, con
     for (int r = 0; r < NR; ++r)
         if (k > 0) zr[r] = T2{zr[r].x + bt * pr[r].x, zr[r].y + bt * pr[r].y};
     DotAcc<T> pq;
-    if (j0 < g.ny) {
+    if (strip) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int j = j0 + r;
@@ -330,7 +333,8 @@ __global__ void __launch_bounds__(128) k_axpy4(Grid g, T *__restrict__ e, T *__r
     const int m = blockIdx.z;
     const int i = 4 * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
     const long long c = (long long)m * g.S + (long long)j * g.P + i;
-    const bool in = i < g.nx;                                // nx % 4 == 0: all four values in
+    // nx % 4 == 0: all four values in; a strip without a fluid cell stays zero
+    const bool in = i < g.nx && g.strips[(j >> 2) * ((g.nx + 63) >> 6) + (i >> 6)];
     // the data first (none of it depends on the control word or on alpha)
     T2 ev[2], rv[2], pv[2], qv[2];
 #pragma unroll
@@ -405,6 +409,9 @@ struct SmoothArgs {
     int order;            // 0: red then black; 1: black then red
     int flags;
     int k;                // inner iteration (for the dot slot)
+    // level 0 in a solve: per tile whether it holds a fluid cell; nullptr: f may be nonzero in solid cells
+    // (envar_apply_preconditioner), every tile runs
+    const uint8_t *tiles;
 };
 
 // Thread layout: a block of 384 threads covers a 64 x 42 region (tile + halo); each thread owns a
@@ -604,6 +611,13 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_smoothw(SmoothArgs sa, const 
     // member does, and the loads of the others would be spent for nothing)
     if (ctl[m].outer_done) return;
     if (inner_guard && ctl[m].inner_done) return;
+    if (sa.tiles && !sa.tiles[blockIdx.x + gridDim.x * blockIdx.y]) {
+        // all solid: the iterate, the restricted residual and the dot product are zero, and the arrays
+        // hold zeros from the start
+        if (sa.flags & (SF_DOT | SF_INIT_DOT))
+            write_block_partial(rc, (sa.flags & SF_INIT_DOT) ? rz_slot(0) : rz_slot(sa.k + 1), m, DotAcc<T>().total());
+        return;
+    }
     const Level &L = sa.L;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i0 = blockIdx.x * TW, j0 = blockIdx.y * TH;
@@ -639,6 +653,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_smoothw(SmoothArgs sa, const 
     auto kN = [&](unsigned int q) { return tab[16 + ((q >> 12) & 15u)]; };
 
     T e0[R], e1[R], f0[R], f1[R], v0[R], v1[R];
+    unsigned int open = 0u;
     // level 0: 8 open bits (two cells) per row, 4 rows per word; CODED: both cells' codes per row
     constexpr int NB = CODED ? R : (R + 3) / 4;
     unsigned int bits[NB];
@@ -687,7 +702,9 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_smoothw(SmoothArgs sa, const 
         v1[r] = (ring_row || lane == 31) ? (T)0 : ir;
         f0[r] = fv.x; f1[r] = fv.y;
         e0[r] = ev.x; e1[r] = ev.y;
+        open |= qq;
     }
+    open = __any_sync(0xffffffffu, open != 0u);                 // a warp of solid cells has nothing to sweep
     xb[1][w][0][lane] = T2{e0[0], e1[0]};
     xb[1][w][1][lane] = T2{e0[R - 1], e1[R - 1]};
     __syncthreads();
@@ -699,6 +716,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_smoothw(SmoothArgs sa, const 
         const int rbuf = (s & 1) ^ 1, wbuf = s & 1;
         const T2 below = xb[rbuf][wb][1][lane];                  // top row of the warp below
         const T2 above = xb[rbuf][wa][0][lane];                  // bottom row of the warp above
+        if (open) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             // the left cell (even column) of row r has colour r & 1 (gj0 and w R are even)
@@ -723,6 +741,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_smoothw(SmoothArgs sa, const 
                     e1[r] = v1[r] * (f1[r] + cx * (e0[r] + eE) + cy * (sS + sN));
                 }
             }
+        }
         }
         xb[wbuf][w][0][lane] = T2{e0[0], e1[0]};
         xb[wbuf][w][1][lane] = T2{e0[R - 1], e1[R - 1]};
@@ -1060,6 +1079,9 @@ static void launch_smoothw(int M, int nsweep, cudaStream_t st, const SmoothArgs 
     count_launches(1);
 }
 
+// sweep pairs that launch_smooth's kernels run for nsweep
+static int smooth_pairs(int nsweep) { return nsweep == 1 ? 1 : nsweep == 2 ? 2 : 3; }
+
 template <class T>
 static void launch_smooth(int M, int nsweep, cudaStream_t st, const SmoothArgs &sa, const T *f, const T *ein, T *e,
                           const T *ec, T *fc, const RedCtx &rc, MemberCtl *ctl, int inner_guard)
@@ -1119,6 +1141,18 @@ template <class T> int rz_parts(const Level &L0, int nu)
     }
     return cdiv(L0.nx, sc_tw(nu)) * cdiv(L0.ny, sc_th(nu));
 }
+// Whether each of the warp-row smoother's level-0 tiles at 1, 2, 3 sweep pairs holds a fluid cell.
+std::vector<uint8_t> smooth_tiles(int nx, int ny, int P, const uint8_t *fluid, bool mixed, int pairs)
+{
+    const int H = s0_halo(pairs), TW = S0_COLS - 2 * H, TH = 12 * (mixed ? S0<float>::R : S0<double>::R) - 2 * H, nt = cdiv(nx, TW);
+    std::vector<uint8_t> t((size_t)nt * cdiv(ny, TH), 0);
+    for (int j = 0; j < ny; ++j)
+        for (int k = 0; k < nt; ++k) {
+            uint8_t &q = t[(size_t)(j / TH) * nt + k];
+            q = q || std::memchr(fluid + (size_t)j * P + k * TW, 1, std::min(TW, nx - k * TW)) != nullptr;
+        }
+    return t;
+}
 int rz_parts_max(const Level &L0, bool mixed)
 {
     int n = 0;
@@ -1128,7 +1162,7 @@ int rz_parts_max(const Level &L0, bool mixed)
 
 template <class T>
 static void vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B, const PoissonCfg &pc, RedCtx rc,
-                   MemberCtl *ctl, int inner_guard, int k, int init, cudaStream_t st)
+                   MemberCtl *ctl, int inner_guard, int k, int init, bool in_solve, cudaStream_t st)
 {
     // level 0 input f = r (inner residual), output z
     const T *f0 = (const T *)B.r;
@@ -1141,7 +1175,7 @@ static void vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B,
         const Level &L = lev[l];
         const Level &Lc = lev[l + 1];
         const int nu = level_sweeps(pc, l, pc.nu_pre);
-        SmoothArgs sa{L, Lc.P, Lc.S, nu, 0, SF_ZERO_INIT | SF_RESTRICT, k};
+        SmoothArgs sa{L, Lc.P, Lc.S, nu, 0, SF_ZERO_INIT | SF_RESTRICT, k, in_solve && l == 0 ? L.tile_fluid[smooth_pairs(nu) - 1] : nullptr};
         const T *f = (l == 0) ? f0 : (const T *)B.lev_f[l];
         T *et = (T *)B.lev_t[l];     // pre-smoothed guess, read by the post-smoothing below
         launch_smooth<T>(M, nu, st, sa, f, (const T *)nullptr, et, (const T *)nullptr, (T *)B.lev_f[l + 1], rc,
@@ -1165,7 +1199,7 @@ static void vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B,
         int flags = SF_PROLONG;
         if (l == 0) flags |= init ? SF_INIT_DOT : SF_DOT;
         const int nu = level_sweeps(pc, l, pc.nu_post);
-        SmoothArgs sa{L, Lc.P, Lc.S, nu, 1, flags, k};
+        SmoothArgs sa{L, Lc.P, Lc.S, nu, 1, flags, k, in_solve && l == 0 ? L.tile_fluid[smooth_pairs(nu) - 1] : nullptr};
         const T *f = (l == 0) ? f0 : (const T *)B.lev_f[l];
         T *e = (l == 0) ? z : (T *)B.lev_e[l];
         launch_smooth<T>(M, nu, st, sa, f, (const T *)B.lev_t[l], e, (const T *)B.lev_e[l + 1], (T *)nullptr,
@@ -1182,7 +1216,7 @@ void launch_vcycle(const Grid &g, const Level *lev, int M, const PoissonBufs &B,
                    const Partials &pt, MemberCtl *ctl, cudaStream_t st)
 {
     RedCtx rc = make_ctx(pt);
-    vcycle<TM>(g, lev, M, B, pc, rc, ctl, 0, 0, 1, st);
+    vcycle<TM>(g, lev, M, B, pc, rc, ctl, 0, 0, 1, false, st);
 }
 template void launch_vcycle<float>(const Grid &, const Level *, int, const PoissonBufs &, const PoissonCfg &,
                                    const Partials &, MemberCtl *, cudaStream_t);
@@ -1257,7 +1291,7 @@ static void refinement(const Grid &g, const Level *lev, int M, const PoissonBufs
     const Level &L0 = lev[0];
     TM *r = (TM *)B.r, *e = (TM *)B.e, *z = (TM *)B.z, *q = (TM *)B.q;
     TM *pv[2] = {(TM *)B.pv, (TM *)B.pv1};
-    vcycle<TM>(g, lev, M, B, pc, rc, ctl, 0, 0, 1, st);
+    vcycle<TM>(g, lev, M, B, pc, rc, ctl, 0, 0, 1, true, st);
     for (int k = 0; k < pc.max_inner; ++k) {
         launch_spmv<TM>(g, L0, M, z, pv[k & 1], pv[(k + 1) & 1], q, rc, ctl, k, st);
         count_launches(1);
@@ -1269,7 +1303,7 @@ static void refinement(const Grid &g, const Level *lev, int M, const PoissonBufs
         launch_axpy<TM>(g, M, e, r, pv[(k + 1) & 1], q, rc, ctl, k, st);
         count_launches(1);
         if (k + 1 == pc.max_inner) break;   // the last update needs no new preconditioned residual
-        vcycle<TM>(g, lev, M, B, pc, rc, ctl, 1, k, 0, st);   // also decides inner convergence
+        vcycle<TM>(g, lev, M, B, pc, rc, ctl, 1, k, 0, true, st);   // also decides inner convergence
     }
     if (pc.df_outer) {
         return;   // max_inner == 0: nothing to add
@@ -1364,13 +1398,13 @@ int launch_poisson_single(int which, const Grid &g, const Level *lev, int M, con
     TM *pv[2] = {(TM *)B.pv, (TM *)B.pv1};
     switch (which) {
     case 1: {
-        SmoothArgs sa{L0, L1.P, L1.S, pc.nu_pre, 0, SF_ZERO_INIT | SF_RESTRICT, 0};
+        SmoothArgs sa{L0, L1.P, L1.S, pc.nu_pre, 0, SF_ZERO_INIT | SF_RESTRICT, 0, L0.tile_fluid[smooth_pairs(pc.nu_pre) - 1]};
         launch_smooth<TM>(M, pc.nu_pre, st, sa, r, (const TM *)nullptr, (TM *)B.lev_t[0], (const TM *)nullptr,
                           (TM *)B.lev_f[1], rc, ctl, 0);
         return 0;
     }
     case 2: {
-        SmoothArgs sa{L0, L1.P, L1.S, pc.nu_post, 1, SF_PROLONG | SF_DOT, 1};
+        SmoothArgs sa{L0, L1.P, L1.S, pc.nu_post, 1, SF_PROLONG | SF_DOT, 1, L0.tile_fluid[smooth_pairs(pc.nu_post) - 1]};
         launch_smooth<TM>(M, pc.nu_post, st, sa, r, (const TM *)B.lev_t[0], z, (const TM *)B.lev_e[1], (TM *)nullptr,
                           rc, ctl, 0);
         return 0;
