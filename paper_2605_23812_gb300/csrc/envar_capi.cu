@@ -96,8 +96,11 @@ struct envar_handle_s {
     int ngroups = 1;                    // concurrent member groups of the captured step
     cudaStream_t side[ENVAR_MAX_GROUPS] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[ENVAR_MAX_GROUPS] = {};
-    cudaEvent_t ev_solved0 = nullptr;   // member 0's pressure increment is final (group 0)
-    cudaEvent_t ev_corr[ENVAR_MAX_GROUPS] = {};   // a group's correction has read member 0's increment
+    // per copy of member 0's velocity (mixed; FP64: one, its increment itself): it is final (group 0), and a
+    // group's correction has read it
+    cudaEvent_t ev_solved0[REF_SLOTS] = {};
+    cudaEvent_t ev_corr[REF_SLOTS][ENVAR_MAX_GROUPS] = {};
+    float4 *d_ref = nullptr;            // mixed, DOMAIN cost: the copies [REF_SLOTS][S]
     int cimg_bytes = 0;
     ClusterPlan *plan = nullptr, *plan_coarse = nullptr;   // cluster pressure solve / coarse V-cycle
     // reduced-space optimisers (allocated on first use)
@@ -571,7 +574,10 @@ static int alloc_buffers(envar_handle h)
         for (float *q : {ms.ush, ms.usl, ms.vsh, ms.vsl, ms.bh, ms.bl}) CK(cudaMemset(q, 0, sizeof(float) * n0));
         if (h->cfg.guess_extrapolation) DA(ms.xp, n0);
         if (h->cfg.cost_mode == ENVAR_COST_DOMAIN) DA(ms.wf, 6 * n0);
-        if (h->cfg.cost_mode == ENVAR_COST_DOMAIN && h->N > 0) DA(ms.wd, 4 * n0);
+        if (h->cfg.cost_mode == ENVAR_COST_DOMAIN && h->N > 0) {
+            DA(ms.wd, 4 * n0);
+            DA(h->d_ref, REF_SLOTS * (size_t)S);
+        }
         DA(ms.frect, (size_t)M * 2 * h->nrect);
         DA(h->ic.uh, S); DA(h->ic.ul, S); DA(h->ic.vh, S); DA(h->ic.vl, S);
         CK(cudaMemset(h->ic.uh, 0, sizeof(float) * S)); CK(cudaMemset(h->ic.ul, 0, sizeof(float) * S));
@@ -715,7 +721,7 @@ static RefMember ref_member(envar_handle h)
 // predictor and the pressure solve (part 0), the projection correction with the cost accumulation
 // (part 1), and (FP64) the re-centring of the pressure increment, the next step's initial guess
 // (part 2; the mixed path re-centres inside the correction and has no part 2).
-static void enqueue_range(envar_handle h, int M, const MemberView &v, cudaStream_t st, int part)
+static void enqueue_range(envar_handle h, int M, const MemberView &v, cudaStream_t st, int part, int slot = 0)
 {
     const Grid &g = h->g;
     const int want_wf = h->cfg.cost_mode == ENVAR_COST_DOMAIN ? 1 : 0;
@@ -725,8 +731,8 @@ static void enqueue_range(envar_handle h, int M, const MemberView &v, cudaStream
             launch_predict_rhs_mx(g, h->mc, M, v.ms, v.ubc, h->d_inh, h->d_inl, v.ctl, v.pt.red, h->nfluid, st);
             launch_pressure_solve<float>(g, h->lev, M, v.pb, h->pc, v.pt, v.ctl, st);
         } else if (part == 1) {
-            launch_correct_mx(g, h->mc, M, v.ms, h->ms, h->x0, h->y0, want_wf, v.series, v.pt, v.ctl, h->cfg.div_tol,
-                              h->nfluid, st);
+            launch_correct_mx(g, h->mc, M, v.ms, h->d_ref + slot * g.S, h->x0, h->y0, want_wf, v.series, v.pt, v.ctl,
+                              h->cfg.div_tol, h->nfluid, st);
         }
         return;
     }
@@ -747,43 +753,61 @@ static void enqueue_range(envar_handle h, int M, const MemberView &v, cudaStream
 // nsteps time steps of the first M member slots.  With all slots and several member groups, each
 // group's steps form one chain on its side stream (a parallel branch of the captured graph, forked
 // once and joined once), so one group's latency-bound phases overlap another's bandwidth-bound
-// ones and the groups need not meet at every step.  The only coupling is member 0: the corrections
-// of groups 1.. read its pressure increment and predictor (the exact DOMAIN contraction), so they
-// wait for group 0's solve of the same step, and group 0 changes member 0's increment again (the
-// FP64 re-centring, the mixed path's next initial guess) only after every group has read it.
+// ones and the groups need not meet at every step.  The only coupling is member 0, whose velocity the
+// corrections of the other members read (the exact DOMAIN contraction).  MIXED: group 0 leaves a copy
+// after its solve and may run REF_SLOTS steps ahead of the slowest group.  FP64: the corrections of
+// groups 1.. read member 0's pressure increment and predictor themselves, so they wait for group
+// 0's solve of the same step, and group 0 changes the increment again (the re-centring) only after
+// every group has read it.
 static void enqueue_steps(envar_handle h, int M, int nsteps)
 {
     const int G = (M == h->Mall) ? h->ngroups : 1;
+    const bool copies = h->d_ref != nullptr && M > 1;
     if (G <= 1) {
         const MemberView v = member_view(h, 0);
         for (int s = 0; s < nsteps; ++s)
-            for (int part = 0; part < 3; ++part) enqueue_range(h, M, v, h->st, part);
+            for (int part = 0; part < 3; ++part) {
+                if (part == 1 && copies) launch_ref_mx(h->g, h->mc, v.ms, v.ctl, h->d_ref, h->st);
+                enqueue_range(h, M, v, h->st, part);
+            }
         return;
     }
     const bool need_m0 = h->ms.wd != nullptr || h->d_wd != nullptr;
-    const int per = (M + G - 1) / G;
+    const int per = (M + G - 1) / G, slots = h->mixed ? REF_SLOTS : 1;
     int ng = 0;
     while (ng < G && ng * per < M) ++ng;
     cudaEventRecord(h->ev_fork, h->st);
     for (int k = 0; k < ng; ++k) cudaStreamWaitEvent(h->side[k], h->ev_fork, 0);
     for (int s = 0; s < nsteps; ++s) {
+        const int slot = s % slots;
         for (int k = 0; k < ng; ++k) {
             const int m0 = k * per, Mg = std::min(per, M - m0);
             const MemberView v = member_view(h, m0);
-            if (need_m0 && k == 0 && s > 0)   // the previous step's corrections have read member 0
-                for (int q = 1; q < ng; ++q) cudaStreamWaitEvent(h->side[0], h->ev_corr[q], 0);
+            // the corrections of the last step that used the slot have read it
+            auto wait_readers = [&]() {
+                for (int q = 1; q < ng; ++q) cudaStreamWaitEvent(h->side[0], h->ev_corr[slot][q], 0);
+            };
+            if (need_m0 && k == 0 && s > 0 && !h->mixed) wait_readers();
             enqueue_range(h, Mg, v, h->side[k], 0);
             if (need_m0) {
-                if (k == 0) cudaEventRecord(h->ev_solved0, h->side[0]);
-                else cudaStreamWaitEvent(h->side[k], h->ev_solved0, 0);
+                if (k == 0) {
+                    if (h->mixed) {
+                        if (s >= slots) wait_readers();
+                        launch_ref_mx(h->g, h->mc, v.ms, v.ctl, h->d_ref + slot * h->g.S, h->side[0]);
+                    }
+                    cudaEventRecord(h->ev_solved0[slot], h->side[0]);
+                } else {
+                    cudaStreamWaitEvent(h->side[k], h->ev_solved0[slot], 0);
+                }
             }
-            enqueue_range(h, Mg, v, h->side[k], 1);
-            if (need_m0 && k > 0) cudaEventRecord(h->ev_corr[k], h->side[k]);
+            enqueue_range(h, Mg, v, h->side[k], 1, slot);
+            if (need_m0 && k > 0) cudaEventRecord(h->ev_corr[slot][k], h->side[k]);
         }
+        if (h->mixed) continue;                              // (no part 2)
         for (int k = 0; k < ng; ++k) {
             const int m0 = k * per, Mg = std::min(per, M - m0);
             if (k == 0 && need_m0)
-                for (int q = 1; q < ng; ++q) cudaStreamWaitEvent(h->side[0], h->ev_corr[q], 0);
+                for (int q = 1; q < ng; ++q) cudaStreamWaitEvent(h->side[0], h->ev_corr[0][q], 0);
             enqueue_range(h, Mg, member_view(h, m0), h->side[k], 2);
         }
     }
@@ -979,12 +1003,15 @@ extern "C" int envar_init(envar_handle *out, const envar_config *cfg, void *cuda
         if (!h->batched) G = 1;
         h->ngroups = std::max(1, std::min(G, h->Mall));
         if (h->ngroups > 1) {
-            bool ok = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
-                      cudaEventCreateWithFlags(&h->ev_solved0, cudaEventDisableTiming) == cudaSuccess;
+            bool ok = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+            for (int r = 0; ok && r < REF_SLOTS; ++r) {
+                ok = cudaEventCreateWithFlags(&h->ev_solved0[r], cudaEventDisableTiming) == cudaSuccess;
+                for (int k = 0; ok && k < h->ngroups; ++k)
+                    ok = cudaEventCreateWithFlags(&h->ev_corr[r][k], cudaEventDisableTiming) == cudaSuccess;
+            }
             for (int k = 0; ok && k < h->ngroups; ++k)
                 ok = cudaStreamCreateWithFlags(&h->side[k], cudaStreamNonBlocking) == cudaSuccess &&
-                     cudaEventCreateWithFlags(&h->ev_join[k], cudaEventDisableTiming) == cudaSuccess &&
-                     cudaEventCreateWithFlags(&h->ev_corr[k], cudaEventDisableTiming) == cudaSuccess;
+                     cudaEventCreateWithFlags(&h->ev_join[k], cudaEventDisableTiming) == cudaSuccess;
             if (!ok) {
                 set_err(nullptr, "envar_init: stream or event creation failed");
                 envar_destroy(h);
@@ -1056,10 +1083,12 @@ extern "C" int envar_destroy(envar_handle h)
     for (int k = 0; k < ENVAR_MAX_GROUPS; ++k) {
         if (h->side[k]) cudaStreamDestroy(h->side[k]);
         if (h->ev_join[k]) cudaEventDestroy(h->ev_join[k]);
-        if (h->ev_corr[k]) cudaEventDestroy(h->ev_corr[k]);
+        for (int r = 0; r < REF_SLOTS; ++r)
+            if (h->ev_corr[r][k]) cudaEventDestroy(h->ev_corr[r][k]);
     }
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
-    if (h->ev_solved0) cudaEventDestroy(h->ev_solved0);
+    for (int r = 0; r < REF_SLOTS; ++r)
+        if (h->ev_solved0[r]) cudaEventDestroy(h->ev_solved0[r]);
     if (h->own_stream) cudaStreamDestroy(h->st);
     delete h;
     return ENVAR_OK;
@@ -1880,7 +1909,7 @@ extern "C" int envar_time_kernel(envar_handle h, int which, int reps, double *ms
             return 0;
         case 6:
             if (h->mixed) {
-                launch_correct_mx(g, h->mc, M, h->ms, h->ms, h->x0, h->y0, wf, ser, h->pt, h->d_ctl, h->cfg.div_tol,
+                launch_correct_mx(g, h->mc, M, h->ms, h->d_ref, h->x0, h->y0, wf, ser, h->pt, h->d_ctl, h->cfg.div_tol,
                                   h->nfluid, h->st);
                 return 0;
             }

@@ -425,8 +425,11 @@ int outer_residual_parts_mx(const Grid &g);
 // The last inner CG update fused with the refinement's x += e (df64 x).
 void launch_axpy_last_mx(const Grid &g, int M, const MixState &s, const float *e, const float *p, const RedCtx &rc,
                          MemberCtl *ctl, int k, cudaStream_t st);
-// ref: member 0's slot (its u*, v* and increment x are read for the Welford of d = u - u_0).
-void launch_correct_mx(const Grid &g, const MixConst &K, int M, const MixState &s, const MixState &ref, double x0,
+// ref: member 0's corrected cell-centred velocity of the same step (launch_ref_mx), read for the Welford
+// of d = u - u_0 where s.wd is given.
+constexpr int REF_SLOTS = 4;
+void launch_ref_mx(const Grid &g, const MixConst &K, const MixState &s, const MemberCtl *ctl, float4 *ref, cudaStream_t st);
+void launch_correct_mx(const Grid &g, const MixConst &K, int M, const MixState &s, const float4 *ref, double x0,
                        double y0, int want_welford, double *series, const Partials &pt, MemberCtl *ctl,
                        double div_tol, long long nfluid, cudaStream_t st);
 // Per-member partial sums over fluid cells of a df64 plane pair (hi, lo) with member stride mstride.

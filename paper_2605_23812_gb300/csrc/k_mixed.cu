@@ -609,7 +609,35 @@ __device__ __forceinline__ void welford2_diff(float a, float b, int n, float *w,
     w[2 * S + c] = m2.h; w[3 * S + c] = m2.l;
 }
 
-__global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixState s, MixState ref, double x0, double y0,
+// Member 0's corrected cell-centred velocity (u, v in df64) in the window, for the difference that every
+// other member accumulates: one 16-byte load there instead of 14 loads and four corrections per cell and
+// member, and the other groups no longer hold up member 0's next step (they read this copy, of
+// which there are REF_SLOTS in turn, not its increment).
+__global__ void __launch_bounds__(256) k_ref_mx(Grid g, MixConst K, MixState s, const MemberCtl *ctl, float4 *__restrict__ ref)
+{
+    const int t = ctl[0].step - (g.n_steps - g.n_window);
+    if (t <= 0 || t > g.n_window) return;
+    const unsigned int tile = g.tiles[blockIdx.x];
+    const int i = (tile & 0xffffu) * 32 + threadIdx.x, j = (tile >> 16) * 8 + threadIdx.y;
+    if (i >= g.nx || j >= g.ny) return;
+    const long long c = (long long)j * g.P + i, cW = c - (i > 0), cS = c - (j > 0 ? g.P : 0);
+    if (!g.fluid[c]) return;
+    const f2 gx{K.gxh, K.gxl}, gy{K.gyh, K.gyl}, xC{s.xh[c], s.xl[c]};
+    const f2 u = corrected(g.uk[c] == FK_UNK, f2{s.ush[c], s.usl[c]}, xC, f2{s.xh[cW], s.xl[cW]}, gx);
+    const f2 uE = corrected(g.uk[c + 1] == FK_UNK, f2{s.ush[c + 1], s.usl[c + 1]}, f2{s.xh[c + 1], s.xl[c + 1]}, xC, gx);
+    const f2 v = corrected(g.vk[c] == FK_UNK, f2{s.vsh[c], s.vsl[c]}, xC, f2{s.xh[cS], s.xl[cS]}, gy);
+    const f2 vN = corrected(g.vk[c + g.P] == FK_UNK, f2{s.vsh[c + g.P], s.vsl[c + g.P]}, f2{s.xh[c + g.P], s.xl[c + g.P]}, xC, gy);
+    const f2 a = df_scale_half(df_add(u, uE)), b = df_scale_half(df_add(v, vN));
+    ref[c] = make_float4(a.h, a.l, b.h, b.l);
+}
+
+void launch_ref_mx(const Grid &g, const MixConst &K, const MixState &s, const MemberCtl *ctl, float4 *ref, cudaStream_t st)
+{
+    k_ref_mx<<<g.ntiles, dim3(32, 8), 0, st>>>(g, K, s, ctl, ref);
+    count_launches(1);
+}
+
+__global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixState s, const float4 *__restrict__ ref, double x0, double y0,
                                                     int want_welford, double *__restrict__ series, Partials pt,
                                                     MemberCtl *ctl, double div_tol, long long nfluid)
 {
@@ -673,15 +701,8 @@ __global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixSt
                 const f2 vc = df_scale_half(df_add(vn, vN));
                 welford2_df(uc, vc, t, s.wf + 6 * off, g.S, c);
                 if (s.wd && gm != 0) {
-                    // member 0's corrected cell-centred velocity from its predictor and increment,
-                    // which this kernel does not modify (member 0's own block writes only u, v, p)
-                    const f2 r_x0{ref.xh[c], ref.xl[c]};
-                    const f2 ru = corrected(uk0, f2{ref.ush[c], ref.usl[c]}, r_x0, f2{ref.xh[cW], ref.xl[cW]}, gx);
-                    const f2 ruE = corrected(ukE, f2{ref.ush[cE], ref.usl[cE]}, f2{ref.xh[cE], ref.xl[cE]}, r_x0, gx);
-                    const f2 rv = corrected(vk0, f2{ref.vsh[c], ref.vsl[c]}, r_x0, f2{ref.xh[cS], ref.xl[cS]}, gy);
-                    const f2 rvN = corrected(vkN, f2{ref.vsh[cN], ref.vsl[cN]}, f2{ref.xh[cN], ref.xl[cN]}, r_x0, gy);
-                    const f2 du = df_sub(uc, df_scale_half(df_add(ru, ruE)));
-                    const f2 dv = df_sub(vc, df_scale_half(df_add(rv, rvN)));
+                    const float4 q = ref[c];                 // member 0's
+                    const f2 du = df_sub(uc, f2{q.x, q.y}), dv = df_sub(vc, f2{q.z, q.w});
                     welford2_diff(du.h + du.l, dv.h + dv.l, t, s.wd + 4 * off, g.S, c);
                 }
             }
@@ -702,7 +723,7 @@ __global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixSt
     }
 }
 
-void launch_correct_mx(const Grid &g, const MixConst &K, int M, const MixState &s, const MixState &ref, double x0,
+void launch_correct_mx(const Grid &g, const MixConst &K, int M, const MixState &s, const float4 *ref, double x0,
                        double y0, int want_welford, double *series, const Partials &pt, MemberCtl *ctl,
                        double div_tol, long long nfluid, cudaStream_t st)
 {
