@@ -23,6 +23,7 @@
 // kernel ends.
 #include <algorithm>
 #include <cstring>
+#include <map>
 #include <vector>
 
 #include "df64.cuh"
@@ -132,7 +133,13 @@ struct ClStageArgs {
     int pitch[3];                    // its row length (gathered stages; stage 0: from the slab's width)
     int rp;                          // byte offset of the residual plane handed to the next stage [bh][bw]
     int seq[3];                      // restriction from the level sums its four children in a row (else row pairs)
-    const void *img[3];              // per thread: x-face, y-face conductances and smoothing factors
+    // x-face, y-face conductances and smoothing factors of the threads' blocks, [value][record].  Stage 0:
+    // blocks with equal values share a record (a cavity has a few dozen), so a level's table stays in L1,
+    // where an image per thread is read from L2 at every visit (1024 x 512, 65 members: 86.6 -> 84 ms);
+    // the gathered stages copy an image per thread to shared memory.
+    const void *img[3];
+    const int *kind[3];              // stage 0: each thread's record
+    int nrec[3];
     int simg[2], sfm;                // gathered stages: byte offsets of their copies in shared memory
     const int *fm;                   // per thread: fluid bits of its cells (16 | 4 << 16 | 1 << 20)
 };
@@ -182,7 +189,7 @@ __device__ __forceinline__ unsigned int sa32(int off) { return sptr(sp<unsigned 
 template <class T, int S> struct Ctx {
     int own[3];                      // byte offset of the block's first cell in each level's border plane
     int pitch[3];                    // its row length in bytes
-    int flags, fm;
+    int flags, fm, kind[3];
     int tid, rank, id, nt;           // id: the stage
     // stage 0: remote rows for the pushes, halo barriers, exchange / gather / reduction counters
     unsigned int pushS[3], pushN[3], rbarS, rbarN;
@@ -540,7 +547,7 @@ template <class T, int b, int S>
 __device__ __forceinline__ void load_cond(const ClusterArgs &a, const Ctx<T, S> &c, int k, Cond<T, b> &q)
 {
     const ClStageArgs &st = a.st[c.id];
-    if constexpr (S == 0) q.template load<true>(reinterpret_cast<const T *>(st.img[k]) + c.rank * st.nt + c.tid, st.nt * a.C);
+    if constexpr (S == 0) q.template load<true>(reinterpret_cast<const T *>(st.img[k]) + c.kind[k], st.nrec[k]);
     else q.template load<false>(sp<const T>(st.simg[k]) + c.tid, st.nt);
 }
 
@@ -1054,6 +1061,8 @@ __global__ void __launch_bounds__(ClLimit<T, B>::threads, 1) k_cluster(const __g
     const unsigned int fl = (unsigned int)rec.y >> 16;
     const bool act = (c.flags & CF_ACT) != 0;
     c.fm = act ? a.st[0].fm[rank * a.nt + tid] : 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c.kind[k] = (B >> k) && (k > 0 || !FIRST) ? a.st[0].kind[k][rank * a.nt + tid] : 0;
     {
         const ClSlab s = a.slab[rank];
         c.rxS = s.rxS; c.rxN = s.rxN;
@@ -1383,33 +1392,40 @@ static bool cut_rows(const std::vector<int> &cnt, const std::vector<int> &x0, co
     return true;
 }
 
+// The B x B blocks of a level that hold fluid, and each block row's count and extent.
+struct ClBlocks {
+    int B, bw, bh, nact = 0;
+    std::vector<uint8_t> act;
+    std::vector<int> cnt, x0, x1;
+    ClBlocks(const ClusterHostLevel &L, int B_) : B(B_), bw(L.nx / B_), bh(L.ny / B_)
+    {
+        act.assign((size_t)bw * bh, 0);
+        cnt.assign(bh, 0); x0.assign(bh, 1 << 30); x1.assign(bh, -1);
+        for (int j = 0; j < bh * B; ++j)
+            for (int i = 0; i < bw * B; ++i)
+                if (L.F[(size_t)j * L.P + i]) act[(size_t)(j / B) * bw + i / B] = 1;
+        for (int y = 0; y < bh; ++y)
+            for (int x = 0; x < bw; ++x)
+                if (act[(size_t)y * bw + x]) { ++cnt[y]; x0[y] = std::min(x0[y], x); x1[y] = x; }
+        for (int c : cnt) nact += c;
+    }
+    bool operator()(int x, int y) const { return x >= 0 && y >= 0 && x < bw && y < bh && act[(size_t)y * bw + x]; }
+};
+
 // Build the plan for the levels from la with B x B blocks on C thread blocks.  Returns a device
 // allocation list through `alloc`; nullptr when the grid does not fit the scheme.
 template <class T>
-static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, int la, int B, int C, const ClusterAlloc &alloc)
+static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, int la, const ClBlocks &bl, int C, const ClusterAlloc &alloc)
 {
-    const int nloc = B == 4 ? 3 : 2;
+    const int B = bl.B, nloc = B == 4 ? 3 : 2, bw = bl.bw, bh = bl.bh;
     if (la + nloc >= nlev) return nullptr;                   // the coarsest level is in a gathered stage
     const ClusterHostLevel &L = hl[la];
-    if (L.nx % B || L.ny % B) return nullptr;
-    const int bw = L.nx / B, bh = L.ny / B;
-    if (bw > 32767 || bh > 32767) return nullptr;
-    auto active = [&](int x, int y) {
-        if (x < 0 || y < 0 || x >= bw || y >= bh) return false;
-        for (int r = 0; r < B; ++r)
-            for (int i = 0; i < B; ++i)
-                if (L.F[(size_t)(y * B + r) * L.P + x * B + i]) return true;
-        return false;
-    };
-    std::vector<int> cnt(bh, 0), x0(bh, 1 << 30), x1(bh, -1), first;
-    int nact = 0;
-    for (int y = 0; y < bh; ++y) {
-        for (int x = 0; x < bw; ++x)
-            if (active(x, y)) { ++cnt[y]; x0[y] = std::min(x0[y], x); x1[y] = x; }
-        nact += cnt[y];
-    }
-    const int limit = B == 4 ? ClLimit<T, 4>::threads : ClLimit<T, 2>::threads;
-    if (!cut_rows(cnt, x0, x1, C, B, limit, 96.0 * 1024 / sizeof(T), &first)) return nullptr;
+    if (L.nx % B || L.ny % B || bw > 32767 || bh > 32767) return nullptr;
+    const std::vector<int> &cnt = bl.cnt, &x0 = bl.x0, &x1 = bl.x1;
+    const int nact = bl.nact, limit = B == 4 ? ClLimit<T, 4>::threads : ClLimit<T, 2>::threads;
+    std::vector<int> first;
+    if (nact > limit * C || !cut_rows(cnt, x0, x1, C, B, limit, 96.0 * 1024 / sizeof(T), &first)) return nullptr;
+    auto active = [&](int x, int y) { return bl(x, y); };
     int most = 1;
     for (int k = 0; k < C; ++k) {
         int c = 0;
@@ -1583,9 +1599,30 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
                         fm[t] |= (H.F[cc] ? 1 : 0) << (sh + r * b + i);
                     }
             }
+            size_t nr = n;
+            if (s == 0) {                                    // merge equal records
+                std::map<std::vector<T>, int> seen;
+                std::vector<int> kind(n);
+                std::vector<T> r((size_t)nc + nv);
+                for (int t = 0; t < n; ++t) {
+                    bool same = t > 0;                       // as the neighbour's, mostly
+                    for (size_t w = 0; w < r.size(); ++w) {
+                        same = same && r[w] == im[w * n + t];
+                        r[w] = im[w * n + t];
+                    }
+                    kind[t] = same ? kind[t - 1] : seen.emplace(r, (int)seen.size()).first->second;
+                }
+                nr = seen.size();
+                im.assign(r.size() * nr, (T)0);
+                for (const auto &q : seen)
+                    for (size_t w = 0; w < r.size(); ++w) im[w * nr + q.second] = q.first[w];
+                st.kind[k] = (const int *)put(kind.data(), kind.size() * sizeof(int));
+                if (!st.kind[k]) return fail();
+            }
+            st.nrec[k] = (int)nr;
             T *d = (T *)put(im.data(), im.size() * sizeof(T));
             if (!d) return fail();
-            k_cluster_factor<<<64, 256, 0, alloc.st>>>(d + (size_t)nc * n, (long long)nv * n, lev >= ncoarse ? 1 : 0);
+            k_cluster_factor<<<64, 256, 0, alloc.st>>>(d + (size_t)nc * nr, (long long)nv * nr, lev >= ncoarse ? 1 : 0);
             count_launches(1);
             st.img[k] = d;
         }
@@ -1638,27 +1675,30 @@ ClusterPlan *cluster_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, boo
     // and the precision alone, so a member's arithmetic does not depend on how many run beside it.
     struct Cand { int B, C; };
     std::vector<Cand> cand;
+    const ClBlocks b2(hl[la], 2), b4(hl[la], 4);
     if (mixed) {
         if (la == 0) cand.push_back({2, 1});
-        for (int C : {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 16}) cand.push_back({4, C});
+        // The smallest cluster that holds the grid, rounded up to the largest size of which as many are
+        // resident (clusters at 180 KB per block, measured: 2: 76, 3 and 4: 36, 5: 28, 6: 23, 7 to 9: 15,
+        // 10: 13, 12: 8, 14 and 16: 7): more SMs per member that no other member could use (256 x 128, 33
+        // members: 3 blocks 8.1 ms, 4 blocks 7.5 ms, 5 blocks 7.9 ms).
+        for (int C : {1, 2, 4, 3, 5, 6, 9, 8, 7, 10, 12, 14, 16}) cand.push_back({4, C});
     } else if (la == 0) {
         // FP64 issues one warp instruction per scheduler in 64 cycles (0.49 FMA per clock and warp, 1.67 per
-        // SM from four warps on, measured): about four warps per block, on up to ten blocks
-        long long blocks = 0;
-        for (int y = 0; y + 1 < hl[0].ny; y += 2)
-            for (int x = 0; x + 1 < hl[0].nx; x += 2)
-                blocks += hl[0].F[(size_t)y * hl[0].P + x] || hl[0].F[(size_t)y * hl[0].P + x + 1] ||
-                          hl[0].F[(size_t)(y + 1) * hl[0].P + x] || hl[0].F[(size_t)(y + 1) * hl[0].P + x + 1];
-        const int want = (int)std::min<long long>(10, std::max<long long>(1, (blocks + 127) / 128));
+        // SM from four warps on, measured): about four warps per block, on up to twelve blocks (256 x 128, 17
+        // members: 10 blocks 10.7 ms, 12 blocks 9.9 ms, 14 blocks 16.2 ms: one block per SM; 128 x 64, one
+        // member: 53.1, 51.8 and 51.8 ms)
+        const int four = std::max(1, cdiv(b2.nact, 128)), want = four > 10 ? 12 : four;
         // up to 256 threads of 2 x 2 cells; beyond, 4 x 4 (three levels stay distributed)
-        if (blocks <= 2560)
+        if (b2.nact <= 2560)
             for (int C = want; C <= CL_MAXC; ++C) cand.push_back({2, C});
         for (int C = want; C <= CL_MAXC; ++C) cand.push_back({4, C});
         for (int C = want; C <= CL_MAXC; ++C) cand.push_back({2, C});
         for (int C = want - 1; C >= 1; --C) cand.push_back({2, C});
     }
     for (const Cand &q : cand) {
-        ClusterPlan *p = mixed ? make_plan<float>(hl, nlev, ncoarse, la, q.B, q.C, alloc) : make_plan<double>(hl, nlev, ncoarse, la, q.B, q.C, alloc);
+        const ClBlocks &bl = q.B == 2 ? b2 : b4;
+        ClusterPlan *p = mixed ? make_plan<float>(hl, nlev, ncoarse, la, bl, q.C, alloc) : make_plan<double>(hl, nlev, ncoarse, la, bl, q.C, alloc);
         if (!p) continue;
         int active = 0;
         SolveArgs sa{};
