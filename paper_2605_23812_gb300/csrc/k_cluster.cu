@@ -141,6 +141,7 @@ struct ClStageArgs {
     const int *kind[3];              // stage 0: each thread's record
     int nrec[3];
     int simg[2], sfm;                // gathered stages: byte offsets of their copies in shared memory
+    int wide, ni, fo;                // a coarsest level of more cells than threads; cells in img; byte offset of f
     const int *fm;                   // per thread: fluid bits of its cells (16 | 4 << 16 | 1 << 20)
 };
 struct ClusterArgs {
@@ -683,6 +684,51 @@ template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a
     }
 }
 
+// A coarsest level of more cells than the block has threads (an odd level of a large grid: 672 x 400 ends
+// at 42 x 25): iterate, right-hand side and conductances in shared memory, the cells of a colour dealt
+// out to the threads.  Without it such a grid runs the levels from 1 on as eight launches per V-cycle.
+template <class T> __device__ __forceinline__ void gathered_wide(const ClusterArgs &a, int tid)
+{
+    const ClStageArgs &st = a.st[1], &up = a.st[0];
+    const int bw = st.bw, nt = st.nt, ni = st.ni, pitch = st.pitch[0], seq = up.seq[up.nlev - 1];
+    T *f = sp<T>(st.fo), *e = sp<T>(st.plane[0]) + pitch + CL_PAD;
+    const T *im = sp<const T>(st.simg[0]), *rp = sp<const T>(up.rp);
+    for (int q = tid; q < bw * st.bh; q += nt) {
+        const int y = (int)__umulhi((unsigned int)q, st.rbw), x = q - y * bw;
+        const T *lo = rp + 2 * y * up.bw + 2 * x, *hi = lo + up.bw;
+        f[q] = sum4(lo[0], lo[1], hi[0], hi[1], seq);
+        e[y * pitch + x] = (T)0;
+    }
+    stage_sync<1>(1, nt);
+    const int hw = (bw + 1) / 2;                             // at most one cell of a colour per pair of columns
+    const unsigned int rhw = 0xffffffffu / (unsigned int)hw + 1u;
+    auto half = [&](int col, bool zero) {
+        for (int q = tid; q < hw * st.bh; q += nt) {
+            const int y = (int)__umulhi((unsigned int)q, rhw), x = 2 * (q - y * hw) + ((y ^ col) & 1);
+            if (x < bw) {
+                const int at = y * bw + x;
+                T *c = e + y * pitch + x;
+                T acc = f[at];
+                if (!zero) {
+                    acc = fma_(im[at], c[-1], acc);
+                    acc = fma_(im[ni + at], c[1], acc);
+                    acc = fma_(im[2 * ni + at], c[-pitch], acc);
+                    acc = fma_(im[3 * ni + at], c[pitch], acc);
+                }
+                *c = im[4 * ni + at] * acc;
+            }
+        }
+        stage_sync<1>(1, nt);
+    };
+    for (int h = 0; h < 2 * a.coarse_sweeps; ++h) half(h & 1, h == 0);
+    for (int h = 0; h < 2 * a.coarse_sweeps; ++h) half((h & 1) ^ 1, false);
+}
+template <class T> __device__ __forceinline__ void gathered_any(const ClusterArgs &a, int tid, int *fail)
+{
+    if (sizeof(T) == 4 && a.st[1].wide) gathered_wide<T>(a, tid);
+    else gathered<T>(a, tid, fail);
+}
+
 // hand the residual of the cluster's last level to the gathered stages and return the coarse
 // correction of this thread's cell
 template <class T, bool MULTI> __device__ __forceinline__ T gather_stage(const ClusterArgs &a, Ctx<T, 0> &c, T res)
@@ -701,7 +747,7 @@ template <class T, bool MULTI> __device__ __forceinline__ T gather_stage(const C
         if (c.rank == 0 && c.tid < nx.nt) {
             mb_wait(gbar, ph, c.fail);
             __syncwarp();
-            gathered<T>(a, c.tid, c.fail);
+            gathered_any<T>(a, c.tid, c.fail);
             stage_sync<1>(1, nx.nt);
             if (c.tid < a.C) {
                 asm volatile("fence.acq_rel.cluster;" ::: "memory");
@@ -716,7 +762,7 @@ template <class T, bool MULTI> __device__ __forceinline__ T gather_stage(const C
     } else {
         if (act) *sp<T>(at) = res;
         __syncthreads();
-        if (c.tid < nx.nt) gathered<T>(a, c.tid, c.fail);
+        if (c.tid < nx.nt) gathered_any<T>(a, c.tid, c.fail);
         __syncthreads();
         return act ? *sp<const T>(from) : (T)0;
     }
@@ -1041,10 +1087,10 @@ __global__ void __launch_bounds__(ClLimit<T, B>::threads, 1) k_cluster(const __g
         for (int s = 1; s < a.nst; ++s) {
             const ClStageArgs &st = a.st[s];
             for (int k = 0; k < st.nlev; ++k) {
-                const int n = (st.B >> k) == 2 ? 16 * st.nt : 5 * st.nt;
+                const int n = (st.B >> k) == 2 ? 16 * st.ni : 5 * st.ni;
                 for (int q = tid; q < n; q += blockDim.x) sp<T>(st.simg[k])[q] = reinterpret_cast<const T *>(st.img[k])[q];
             }
-            for (int q = tid; q < st.nt; q += blockDim.x) sp<int>(st.sfm)[q] = st.fm[q];
+            for (int q = tid; q < st.ni; q += blockDim.x) sp<int>(st.sfm)[q] = st.fm[q];
         }
     if (FIRST && tid < 16) {
         const unsigned int q = tid;
@@ -1451,6 +1497,11 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
         s.B = q; s.nlev = q; s.l0 = l; s.bw = hl[l].nx / q; s.bh = hl[l].ny / q;
         s.nt = round_up(s.bw * s.bh, 32);
         s.rbw = 0xffffffffu / (unsigned int)s.bw + 1u;
+        s.ni = s.nt;
+        if (la > 0 && ns == 1 && s.nlev == 1 && l + 1 == nlev && s.nt > nt && s.nt <= 4 * nt) {
+            s.wide = 1;
+            s.nt = nt;
+        }
         if (s.nt > nt || s.bw < 2) return fail();
         l += s.nlev;
         ++ns;
@@ -1510,10 +1561,12 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
     for (int s = 1; s < ns; ++s) {
         for (int k = 0; k < a.st[s].nlev; ++k) {
             a.st[s].simg[k] = (int)o;
-            o = up16(o + sizeof(T) * ((a.st[s].B >> k) == 2 ? 16 : 5) * (size_t)a.st[s].nt);
+            o = up16(o + sizeof(T) * ((a.st[s].B >> k) == 2 ? 16 : 5) * (size_t)a.st[s].ni);
         }
         a.st[s].sfm = (int)o;
-        o = up16(o + sizeof(int) * (size_t)a.st[s].nt);
+        o = up16(o + sizeof(int) * (size_t)a.st[s].ni);
+        a.st[s].fo = (int)o;
+        if (a.st[s].wide) o = up16(o + sizeof(T) * (size_t)a.st[s].ni);
     }
     a.sm_lut = (int)o; o = up16(o + 32 * sizeof(T));
     a.sm_red = (int)o; o = up16(o + 32 * 8);
@@ -1563,7 +1616,7 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
     if (!a.rec) return fail();
     for (int s = 0; s < ns; ++s) {
         ClStageArgs &st = a.st[s];
-        const int n = s == 0 ? C * nt : st.nt;
+        const int n = s == 0 ? C * nt : st.ni;
         std::vector<int> fm(n, 0);
         auto block = [&](int t, int *x, int *y) {
             if (s == 0) {
