@@ -133,14 +133,15 @@ struct ClStageArgs {
     int pitch[3];                    // its row length (gathered stages; stage 0: from the slab's width)
     int rp;                          // byte offset of the residual plane handed to the next stage [bh][bw]
     int seq[3];                      // restriction from the level sums its four children in a row (else row pairs)
-    // x-face, y-face conductances and smoothing factors of the threads' blocks, [value][record].  Stage 0:
-    // blocks with equal values share a record (a cavity has a few dozen), so a level's table stays in L1,
-    // where an image per thread is read from L2 at every visit (1024 x 512, 65 members: 86.6 -> 84 ms);
-    // the gathered stages copy an image per thread to shared memory.
+    // x-face, y-face conductances and smoothing factors of the threads' blocks, [value][record], copied to
+    // shared memory (FP64, stage 0: left in global memory, for a second block per SM).  Stage 0: blocks with
+    // equal values share a record (a cavity has a few dozen), so the tables fit: the V-cycle of 14 members at
+    // 1024 x 512 took 53 us with the tables in L1, 45 us with them in shared memory.  Gathered stages: an
+    // image per thread.
     const void *img[3];
     const int *kind[3];              // stage 0: each thread's record
     int nrec[3];
-    int simg[2], sfm;                // gathered stages: byte offsets of their copies in shared memory
+    int simg[3], sfm;                // gathered stages: byte offsets of their copies in shared memory
     int wide, ni, fo;                // a coarsest level of more cells than threads; cells in img; byte offset of f
     const int *fm;                   // per thread: fluid bits of its cells (16 | 4 << 16 | 1 << 20)
 };
@@ -348,35 +349,30 @@ template <class T, int b> struct Cond {
     __device__ __forceinline__ T x(int r, int i) const { return x_[r][i]; }
     __device__ __forceinline__ T y(int r, int i) const { return y_[r][i]; }
     __device__ __forceinline__ T v(int r, int i) const { return v_[r][i]; }
-    // img: [value][thread], stride threads; GLOBAL: in global memory, else its copy in shared memory
-    template <bool GLOBAL> __device__ __forceinline__ void load(const T *img, int stride)
+    // img: [value][record], n records
+    __device__ __forceinline__ void load(const T *img, int n)
     {
         const T *q = img;
-        auto ld = [](const T *p) {
-            if constexpr (GLOBAL) return __ldg(p);
-            else return *p;
-        };
 #pragma unroll
         for (int r = 0; r < b; ++r)
 #pragma unroll
-            for (int i = 0; i <= b; ++i, q += stride) x_[r][i] = ld(q);
+            for (int i = 0; i <= b; ++i, q += n) x_[r][i] = *q;
 #pragma unroll
         for (int r = 0; r <= b; ++r)
 #pragma unroll
-            for (int i = 0; i < b; ++i, q += stride) y_[r][i] = ld(q);
+            for (int i = 0; i < b; ++i, q += n) y_[r][i] = *q;
 #pragma unroll
         for (int r = 0; r < b; ++r)
 #pragma unroll
-            for (int i = 0; i < b; ++i, q += stride) v_[r][i] = ld(q);
+            for (int i = 0; i < b; ++i, q += n) v_[r][i] = *q;
     }
 };
 template <class T> struct Cond<T, 4> {
-    const T *p;
-    int s;
-    __device__ __forceinline__ T x(int r, int i) const { return __ldg(p + (r * 5 + i) * s); }
-    __device__ __forceinline__ T y(int r, int i) const { return __ldg(p + (20 + r * 4 + i) * s); }
-    __device__ __forceinline__ T v(int r, int i) const { return __ldg(p + (40 + r * 4 + i) * s); }
-    template <bool> __device__ __forceinline__ void load(const T *img, int stride) { p = img; s = stride; }
+    int o, n;                        // byte offset of the record
+    __device__ __forceinline__ T x(int r, int i) const { return sp<const T>(o)[(r * 5 + i) * n]; }
+    __device__ __forceinline__ T y(int r, int i) const { return sp<const T>(o)[(20 + r * 4 + i) * n]; }
+    __device__ __forceinline__ T v(int r, int i) const { return sp<const T>(o)[(40 + r * 4 + i) * n]; }
+    __device__ __forceinline__ void load(const T *img, int n_) { o = (int)(reinterpret_cast<const unsigned char *>(img) - sp<const unsigned char>(0)); n = n_; }
 };
 
 // uniform conductances and open-face bits (the grid's first level)
@@ -548,8 +544,9 @@ template <class T, int b, int S>
 __device__ __forceinline__ void load_cond(const ClusterArgs &a, const Ctx<T, S> &c, int k, Cond<T, b> &q)
 {
     const ClStageArgs &st = a.st[c.id];
-    if constexpr (S == 0) q.template load<true>(reinterpret_cast<const T *>(st.img[k]) + c.kind[k], st.nrec[k]);
-    else q.template load<false>(sp<const T>(st.simg[k]) + c.tid, st.nt);
+    if constexpr (S > 0) q.load(sp<const T>(st.simg[k]) + c.tid, st.nt);
+    else if constexpr (sizeof(T) == 4) q.load(sp<const T>(st.simg[k]) + c.kind[k], st.nrec[k]);
+    else q.load(reinterpret_cast<const T *>(st.img[k]) + c.kind[k], st.nrec[k]);
 }
 
 template <class T, int b, int S, bool MULTI, class Q>
@@ -605,7 +602,7 @@ template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a
     };
     auto cond1 = [&](Cond<T, 1> &q) {
         const ClStageArgs &st = a.st[c.id];
-        q.template load<false>(sp<const T>(st.simg[st.B == 2 ? 1 : 0]) + tid, st.nt);
+        q.load(sp<const T>(st.simg[st.B == 2 ? 1 : 0]) + tid, st.nt);
     };
     int s = 1;
     for (;; ++s) {                                           // down
@@ -1082,16 +1079,16 @@ __global__ void __launch_bounds__(ClLimit<T, B>::threads, 1) k_cluster(const __g
     }
     T *lut = sp<T>(a.sm_lut);
     const T cx = sizeof(T) == 4 ? (T)sa.cxf : (T)sa.cxd, cy = sizeof(T) == 4 ? (T)sa.cyf : (T)sa.cyd;
-    // conductances and fluid bits of the gathered stages
-    if (rank == 0)
-        for (int s = 1; s < a.nst; ++s) {
-            const ClStageArgs &st = a.st[s];
-            for (int k = 0; k < st.nlev; ++k) {
-                const int n = (st.B >> k) == 2 ? 16 * st.ni : 5 * st.ni;
-                for (int q = tid; q < n; q += blockDim.x) sp<T>(st.simg[k])[q] = reinterpret_cast<const T *>(st.img[k])[q];
-            }
-            for (int q = tid; q < st.ni; q += blockDim.x) sp<int>(st.sfm)[q] = st.fm[q];
+    // conductance tables, and the gathered stages' fluid bits
+    for (int s = sizeof(T) == 4 ? 0 : 1; s < (rank == 0 ? a.nst : 1); ++s) {
+        const ClStageArgs &st = a.st[s];
+        for (int k = 0; k < st.nlev; ++k) {
+            const int b = st.B >> k, n = (2 * b * (b + 1) + b * b) * st.nrec[k];
+            for (int q = tid; q < n; q += blockDim.x) sp<T>(st.simg[k])[q] = reinterpret_cast<const T *>(st.img[k])[q];
         }
+        if (s > 0)
+            for (int q = tid; q < st.ni; q += blockDim.x) sp<int>(st.sfm)[q] = st.fm[q];
+    }
     if (FIRST && tid < 16) {
         const unsigned int q = tid;
         const T d = ((q & 1u) ? cx : (T)0) + ((q & 2u) ? cx : (T)0) + ((q & 4u) ? cy : (T)0) + ((q & 8u) ? cy : (T)0);
@@ -1531,54 +1528,6 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
             if (k + 1 < C && active(x, s.rb0 + s.hb - 1) && active(x, s.rb0 + s.hb)) ++s.rxN;
         }
     }
-    // ---- shared memory
-    size_t o = 64;                                           // eight barriers
-    auto up16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
-    for (int k = 0; k < nloc; ++k) {
-        size_t most_b = 0;
-        const int b = B >> k;
-        for (int r = 0; r < C; ++r)
-            most_b = std::max(most_b, (size_t)(a.slab[r].wb * b + 2 * CL_PAD) * (a.slab[r].hb * b + 2));
-        a.st[0].plane[k] = (int)o;
-        o = up16(o + most_b * sizeof(T));
-    }
-    a.st[0].rp = (int)o;
-    o = up16(o + (size_t)bw * bh * sizeof(T));
-    for (int s = 1; s < ns; ++s) {
-        for (int k = 0; k < a.st[s].nlev; ++k) {
-            const int b = a.st[s].B >> k;
-            a.st[s].pitch[k] = a.st[s].bw * b + 2 * CL_PAD + (a.st[s].bw * b) % 2;
-            a.st[s].plane[k] = (int)o;
-            o = up16(o + (size_t)a.st[s].pitch[k] * (a.st[s].bh * b + 2) * sizeof(T));
-        }
-        a.st[s].rp = (int)o;
-        o = up16(o + (size_t)a.st[s].bw * a.st[s].bh * sizeof(T));
-    }
-    // (the planes above are zeroed; everything below is written before it is read)
-    a.sm_idle = (int)o; o += 6 * 128;
-    a.sm_p = (int)o;
-    if (la == 0) o = up16(o + sizeof(T) * B * B * (size_t)nt);
-    for (int s = 1; s < ns; ++s) {
-        for (int k = 0; k < a.st[s].nlev; ++k) {
-            a.st[s].simg[k] = (int)o;
-            o = up16(o + sizeof(T) * ((a.st[s].B >> k) == 2 ? 16 : 5) * (size_t)a.st[s].ni);
-        }
-        a.st[s].sfm = (int)o;
-        o = up16(o + sizeof(int) * (size_t)a.st[s].ni);
-        a.st[s].fo = (int)o;
-        if (a.st[s].wide) o = up16(o + sizeof(T) * (size_t)a.st[s].ni);
-    }
-    a.sm_lut = (int)o; o = up16(o + 32 * sizeof(T));
-    a.sm_red = (int)o; o = up16(o + 32 * 8);
-    a.sm_slot = (int)o; o = up16(o + 2 * CL_MAXC * 8);
-    a.sm_xs = (int)o;
-    if (la == 0 && sizeof(T) == 4) {
-        const int nb = cdiv(L.nx, 64) * cdiv(L.ny, 32);
-        o = up16(o + (size_t)cdiv(nb, C) * 8 * 8);
-    }
-    P->smem = o;
-    P->threads = nt;
-    if (o > 226 * 1024) return fail();
     // ---- per-thread records of stage 0 (blocks of a slab row by row; idle threads at the end)
     struct Th { int x, y; };
     std::vector<std::vector<Th>> th(C);
@@ -1610,14 +1559,13 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
             rec[(size_t)k * nt + t] = int4{x | (y << 16), fg | (int)(fl << 16), (int)ob[0], (int)ob[1]};
         }
     }
-    // ---- per-level conductances, smoothing factors and fluid bits
-    auto put = [&](const void *h, size_t bytes) { return alloc(h, bytes); };
-    a.rec = (const int4 *)put(rec.data(), rec.size() * sizeof(int4));
-    if (!a.rec) return fail();
+    // ---- per-level conductances, smoothing factors (their denominators, here) and fluid bits
+    std::vector<T> table[CL_STAGES][3];
+    std::vector<int> kind[3], fm[CL_STAGES];
     for (int s = 0; s < ns; ++s) {
         ClStageArgs &st = a.st[s];
         const int n = s == 0 ? C * nt : st.ni;
-        std::vector<int> fm(n, 0);
+        fm[s].assign(n, 0);
         auto block = [&](int t, int *x, int *y) {
             if (s == 0) {
                 const int4 q = rec[t];
@@ -1631,8 +1579,7 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
             const int b = st.B >> k, lev = st.l0 + k;
             const ClusterHostLevel &H = hl[lev];
             if (lev == 0) {                                  // uniform conductances: no image
-                for (int t = 0; t < n; ++t) fm[t] = 0;
-                st.img[k] = nullptr;
+                st.nrec[k] = 0;
                 continue;
             }
             const int nc = 2 * b * (b + 1), nv = b * b, sh = b == 4 ? 0 : b == 2 ? 16 : 20;
@@ -1649,37 +1596,100 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
                     for (int i = 0; i < b; ++i, w += n) {
                         const size_t cc = (size_t)(y * b + r) * H.P + x * b + i;
                         im[w] = (((T)H.cw[cc] + (T)H.cw[cc + 1]) + (T)H.cs[cc]) + (T)H.cs[cc + H.P];
-                        fm[t] |= (H.F[cc] ? 1 : 0) << (sh + r * b + i);
+                        fm[s][t] |= (H.F[cc] ? 1 : 0) << (sh + r * b + i);
                     }
             }
             size_t nr = n;
             if (s == 0) {                                    // merge equal records
                 std::map<std::vector<T>, int> seen;
-                std::vector<int> kind(n);
                 std::vector<T> r((size_t)nc + nv);
+                kind[k].resize(n);
                 for (int t = 0; t < n; ++t) {
                     bool same = t > 0;                       // as the neighbour's, mostly
                     for (size_t w = 0; w < r.size(); ++w) {
                         same = same && r[w] == im[w * n + t];
                         r[w] = im[w * n + t];
                     }
-                    kind[t] = same ? kind[t - 1] : seen.emplace(r, (int)seen.size()).first->second;
+                    kind[k][t] = same ? kind[k][t - 1] : seen.emplace(r, (int)seen.size()).first->second;
                 }
                 nr = seen.size();
                 im.assign(r.size() * nr, (T)0);
                 for (const auto &q : seen)
                     for (size_t w = 0; w < r.size(); ++w) im[w * nr + q.second] = q.first[w];
-                st.kind[k] = (const int *)put(kind.data(), kind.size() * sizeof(int));
-                if (!st.kind[k]) return fail();
             }
             st.nrec[k] = (int)nr;
-            T *d = (T *)put(im.data(), im.size() * sizeof(T));
+            table[s][k] = std::move(im);
+        }
+    }
+    // ---- shared memory
+    size_t o = 64;                                           // eight barriers
+    auto up16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
+    for (int k = 0; k < nloc; ++k) {
+        size_t most_b = 0;
+        const int b = B >> k;
+        for (int r = 0; r < C; ++r)
+            most_b = std::max(most_b, (size_t)(a.slab[r].wb * b + 2 * CL_PAD) * (a.slab[r].hb * b + 2));
+        a.st[0].plane[k] = (int)o;
+        o = up16(o + most_b * sizeof(T));
+    }
+    a.st[0].rp = (int)o;
+    o = up16(o + (size_t)bw * bh * sizeof(T));
+    for (int s = 1; s < ns; ++s) {
+        for (int k = 0; k < a.st[s].nlev; ++k) {
+            const int b = a.st[s].B >> k;
+            a.st[s].pitch[k] = a.st[s].bw * b + 2 * CL_PAD + (a.st[s].bw * b) % 2;
+            a.st[s].plane[k] = (int)o;
+            o = up16(o + (size_t)a.st[s].pitch[k] * (a.st[s].bh * b + 2) * sizeof(T));
+        }
+        a.st[s].rp = (int)o;
+        o = up16(o + (size_t)a.st[s].bw * a.st[s].bh * sizeof(T));
+    }
+    // (the planes above are zeroed; everything below is written before it is read)
+    a.sm_idle = (int)o; o += 6 * 128;
+    a.sm_p = (int)o;
+    if (la == 0) o = up16(o + sizeof(T) * B * B * (size_t)nt);
+    for (int s = 0; s < ns; ++s) {
+        for (int k = 0; k < a.st[s].nlev; ++k) {
+            a.st[s].simg[k] = (int)o;
+            if (s > 0 || sizeof(T) == 4) o = up16(o + sizeof(T) * table[s][k].size());
+        }
+        if (s == 0) continue;
+        a.st[s].sfm = (int)o;
+        o = up16(o + sizeof(int) * (size_t)a.st[s].ni);
+        a.st[s].fo = (int)o;
+        if (a.st[s].wide) o = up16(o + sizeof(T) * (size_t)a.st[s].ni);
+    }
+    a.sm_lut = (int)o; o = up16(o + 32 * sizeof(T));
+    a.sm_red = (int)o; o = up16(o + 32 * 8);
+    a.sm_slot = (int)o; o = up16(o + 2 * CL_MAXC * 8);
+    a.sm_xs = (int)o;
+    if (la == 0 && sizeof(T) == 4) {
+        const int nb = cdiv(L.nx, 64) * cdiv(L.ny, 32);
+        o = up16(o + (size_t)cdiv(nb, C) * 8 * 8);
+    }
+    P->smem = o;
+    P->threads = nt;
+    if (o > 226 * 1024) return fail();
+    // ---- uploads
+    auto put = [&](const void *h, size_t bytes) { return alloc(h, bytes); };
+    a.rec = (const int4 *)put(rec.data(), rec.size() * sizeof(int4));
+    if (!a.rec) return fail();
+    for (int s = 0; s < ns; ++s) {
+        ClStageArgs &st = a.st[s];
+        for (int k = 0; k < st.nlev; ++k) {
+            const int b = st.B >> k, lev = st.l0 + k;
+            if (lev == 0) continue;
+            if (s == 0) {
+                st.kind[k] = (const int *)put(kind[k].data(), kind[k].size() * sizeof(int));
+                if (!st.kind[k]) return fail();
+            }
+            T *d = (T *)put(table[s][k].data(), table[s][k].size() * sizeof(T));
             if (!d) return fail();
-            k_cluster_factor<<<64, 256, 0, alloc.st>>>(d + (size_t)nc * nr, (long long)nv * nr, lev >= ncoarse ? 1 : 0);
+            k_cluster_factor<<<4, 256, 0, alloc.st>>>(d + (size_t)2 * b * (b + 1) * st.nrec[k], (long long)b * b * st.nrec[k], lev >= ncoarse ? 1 : 0);
             count_launches(1);
             st.img[k] = d;
         }
-        st.fm = (const int *)put(fm.data(), fm.size() * sizeof(int));
+        st.fm = (const int *)put(fm[s].data(), fm[s].size() * sizeof(int));
         if (!st.fm) return fail();
     }
     return P;
