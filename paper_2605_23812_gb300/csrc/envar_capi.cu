@@ -999,7 +999,10 @@ extern "C" int envar_init(envar_handle *out, const envar_config *cfg, void *cuda
         h->own_stream = true;
     }
     {   // member groups: side streams and fork / join events for the captured step
-        int G = c.member_groups ? c.member_groups : (h->Mall >= 24 ? 4 : (h->Mall >= 8 ? 2 : 1));
+        // small groups pack the cluster solves of one beside the flow kernels of the others: 592 x 240, 17
+        // members: 1, 2, 4, 6, 8 groups 36.8, 25.6, 22.9, 22.7, 22.7 ms; 512 x 256, 33 members: 31.6, 26.0,
+        // 24.5, 24.2, 24.1 ms; 672 x 400, 11 members: 33.5, 29.6, 29.3, 29.1, 29.1 ms
+        int G = c.member_groups ? c.member_groups : (h->Mall >= 8 ? 6 : 1);
         if (!h->batched) G = 1;
         h->ngroups = std::max(1, std::min(G, h->Mall));
         if (h->ngroups > 1) {
