@@ -259,8 +259,8 @@ static int build_geometry(envar_handle h)
     CK(cudaMemcpy(dvk, vk.data(), S, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(duin, uin.data(), sizeof(double) * ny, cudaMemcpyHostToDevice));
     g.fluid = dF; g.uk = duk; g.vk = dvk; g.u_in = duin;
+    std::vector<unsigned int> tiles;
     {
-        std::vector<unsigned int> tiles;
         for (int tj = 0; tj * 8 <= ny; ++tj)
             for (int ti = 0; ti * 32 <= nx; ++ti) {
                 const int i0 = ti * 32, w = std::min(32, nx + 1 - i0);
@@ -484,6 +484,24 @@ static int build_geometry(envar_handle h)
     }
     h->ia = ia; h->ja = ja; h->nrx = ib - ia + 1; h->nry = jb - ja + 1; h->nrect = h->nrx * h->nry;
     g.ia = ia; g.ja = ja; g.nrx = h->nrx; g.nry = h->nry;
+    {
+        std::vector<uint8_t> tf(tiles.size(), 0);
+        const std::vector<uint8_t> ones(35, 1);              // FK_UNK, and the fluid flag
+        for (size_t q = 0; q < tiles.size(); ++q) {
+            const int i0 = (int)(tiles[q] & 0xffffu) * 32, j0 = (int)(tiles[q] >> 16) * 8;
+            bool inner = i0 > 0 && j0 > 0 && i0 + 33 < nx && j0 + 9 < ny;
+            for (int j = j0 - 1; j <= j0 + 9 && inner; ++j) {
+                const size_t c = (size_t)j * P + i0 - 1;
+                inner = !std::memcmp(&uk[c], ones.data(), 35) && !std::memcmp(&vk[c], ones.data(), 35) && !std::memcmp(&F[c], ones.data(), 35);
+            }
+            const bool force = i0 + 32 >= ia && i0 - 1 < ia + h->nrx && j0 + 8 >= ja && j0 - 1 < ja + h->nry;
+            tf[q] = (inner ? TF_INNER : 0) | (force ? TF_FORCE : 0);
+        }
+        uint8_t *d;
+        DA(d, tf.size());
+        CK(cudaMemcpy(d, tf.data(), tf.size(), cudaMemcpyHostToDevice));
+        g.tile_flags = d;
+    }
     std::vector<int> cidx;
     std::vector<uint8_t> rc((size_t)h->nrect, 0);
     for (int j = ja; j <= jb; ++j)

@@ -48,6 +48,8 @@ struct Level {
     const uint8_t *tile_fluid[3];
 };
 
+enum TileFlag : uint8_t { TF_INNER = 1, TF_FORCE = 2 };
+
 struct Grid {
     int nx, ny, P;
     long long S;
@@ -64,6 +66,8 @@ struct Grid {
     // the 32 x 8 tiles (column | row << 16) that hold a fluid cell or a face that is not a wall: the
     // flow kernels visit these alone, walls and solid keep the zeros they start with
     const unsigned int *tiles;
+    const uint8_t *tile_flags;   // TF_INNER: all faces and cells of the tile and one around it are unknowns and fluid;
+                                 // TF_FORCE: the tile or one around it touches the control rectangle
     int ntiles;
     // per 64 x 4 strip of cells, row by row of strips: whether it holds a fluid cell
     const uint8_t *strips;
