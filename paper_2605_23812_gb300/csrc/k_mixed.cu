@@ -48,21 +48,23 @@ void launch_load_ic_mx(const Grid &g, const double *u0, const double *v0, const 
     count_launches(1);
 }
 
-__global__ void k_broadcast4(const float *__restrict__ a, const float *__restrict__ b, const float *__restrict__ c,
-                             const float *__restrict__ d, float *A, float *B, float *C, float *D, long long S, int M)
+// S is a multiple of 32: the planes are copied in 16-byte words (one member per blockIdx.y).
+__global__ void k_broadcast4(const float4 *__restrict__ a, const float4 *__restrict__ b, const float4 *__restrict__ c,
+                             const float4 *__restrict__ d, float4 *A, float4 *B, float4 *C, float4 *D, int S4)
 {
-    long long n = S * (long long)M;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-        long long k = t % S;
-        A[t] = a[k]; B[t] = b[k]; C[t] = c[k]; D[t] = d[k];
-    }
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= S4) return;
+    const long long t = (long long)blockIdx.y * S4 + k;
+    A[t] = a[k]; B[t] = b[k]; C[t] = c[k]; D[t] = d[k];
 }
 
 void launch_reset_mx(const Grid &g, int M, const MixState &ic, const MixState &s, MemberCtl *ctl, int want_welford,
                      cudaStream_t st)
 {
     size_t fb = sizeof(float) * (size_t)g.S * M;
-    k_broadcast4<<<1024, 256, 0, st>>>(ic.uh, ic.ul, ic.vh, ic.vl, s.uh, s.ul, s.vh, s.vl, g.S, M);
+    auto q = [](float *p) { return reinterpret_cast<float4 *>(p); };
+    const int S4 = (int)(g.S / 4);
+    k_broadcast4<<<dim3(cdiv(S4, 256), M), 256, 0, st>>>(q(ic.uh), q(ic.ul), q(ic.vh), q(ic.vl), q(s.uh), q(s.ul), q(s.vh), q(s.vl), S4);
     count_launches(1);
     cudaMemsetAsync(s.p, 0, fb, st);
     cudaMemsetAsync(s.xh, 0, fb, st);
