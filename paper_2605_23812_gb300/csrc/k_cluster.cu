@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <utility>
 #include <vector>
 
 #include "df64.cuh"
@@ -1445,8 +1446,11 @@ struct ClBlocks {
         act.assign((size_t)bw * bh, 0);
         cnt.assign(bh, 0); x0.assign(bh, 1 << 30); x1.assign(bh, -1);
         for (int j = 0; j < bh * B; ++j)
-            for (int i = 0; i < bw * B; ++i)
-                if (L.F[(size_t)j * L.P + i]) act[(size_t)(j / B) * bw + i / B] = 1;
+            for (int x = 0; x < bw; ++x) {
+                unsigned int q = 0;                          // the block's cells of the row (a byte each)
+                std::memcpy(&q, L.F + (size_t)j * L.P + x * B, B);
+                act[(size_t)(j / B) * bw + x] |= q != 0;
+            }
         for (int y = 0; y < bh; ++y)
             for (int x = 0; x < bw; ++x)
                 if (act[(size_t)y * bw + x]) { ++cnt[y]; x0[y] = std::min(x0[y], x); x1[y] = x; }
@@ -1670,28 +1674,35 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
     P->smem = o;
     P->threads = nt;
     if (o > 226 * 1024) return fail();
-    // ---- uploads
-    auto put = [&](const void *h, size_t bytes) { return alloc(h, bytes); };
-    a.rec = (const int4 *)put(rec.data(), rec.size() * sizeof(int4));
-    if (!a.rec) return fail();
+    // ---- one upload
+    std::vector<unsigned char> blob;
+    std::vector<std::pair<const void **, size_t>> at;        // pointers and their places in it
+    auto put = [&](const void **dst, const void *src, size_t bytes) {
+        at.emplace_back(dst, blob.size());
+        blob.resize(up16(blob.size() + bytes));
+        if (bytes) std::memcpy(&blob[at.back().second], src, bytes);
+    };
+    put((const void **)&a.rec, rec.data(), rec.size() * sizeof(int4));
     for (int s = 0; s < ns; ++s) {
         ClStageArgs &st = a.st[s];
         for (int k = 0; k < st.nlev; ++k) {
+            if (st.l0 + k == 0) continue;
+            if (s == 0) put((const void **)&st.kind[k], kind[k].data(), kind[k].size() * sizeof(int));
+            put(&st.img[k], table[s][k].data(), table[s][k].size() * sizeof(T));
+        }
+        put((const void **)&st.fm, fm[s].data(), fm[s].size() * sizeof(int));
+    }
+    const unsigned char *dev = (const unsigned char *)alloc(blob.data(), blob.size());
+    if (!dev) return fail();
+    for (const auto &q : at) *q.first = dev + q.second;
+    for (int s = 0; s < ns; ++s)
+        for (int k = 0; k < a.st[s].nlev; ++k) {
+            const ClStageArgs &st = a.st[s];
             const int b = st.B >> k, lev = st.l0 + k;
             if (lev == 0) continue;
-            if (s == 0) {
-                st.kind[k] = (const int *)put(kind[k].data(), kind[k].size() * sizeof(int));
-                if (!st.kind[k]) return fail();
-            }
-            T *d = (T *)put(table[s][k].data(), table[s][k].size() * sizeof(T));
-            if (!d) return fail();
-            k_cluster_factor<<<4, 256, 0, alloc.st>>>(d + (size_t)2 * b * (b + 1) * st.nrec[k], (long long)b * b * st.nrec[k], lev >= ncoarse ? 1 : 0);
+            k_cluster_factor<<<4, 256, 0, alloc.st>>>((T *)st.img[k] + (size_t)2 * b * (b + 1) * st.nrec[k], (long long)b * b * st.nrec[k], lev >= ncoarse ? 1 : 0);
             count_launches(1);
-            st.img[k] = d;
         }
-        st.fm = (const int *)put(fm[s].data(), fm[s].size() * sizeof(int));
-        if (!st.fm) return fail();
-    }
     return P;
 }
 
