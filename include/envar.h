@@ -104,8 +104,8 @@ typedef struct envar_config {
     int coarse_sweeps;       /* symmetric sweep pairs on the coarsest multigrid level */
     int steps_per_graph;     /* time steps per captured CUDA graph (even) */
     int member_groups;       /* batched runs: member groups whose time steps run as concurrent
-                                branches of the captured graph; 0 = automatic (4 from 24 member
-                                slots, 2 from 8), 1 .. 8 */
+                                branches of the captured graph; 0 = automatic (6 from 8 member
+                                slots on), 1 .. 8 */
     int lip_slip;            /* 1: the lower wall of the channel (y = 0) is free slip outside
                                 noslip_span and no slip inside it (the slip segments of Sec. 4.4);
                                 0: no slip everywhere */
