@@ -156,6 +156,7 @@ struct ClusterArgs {
     int nact;                        // blocks that hold fluid (gathered residuals)
     int sm_p, sm_lut, sm_red, sm_slot, sm_xs;   // byte offsets in shared memory
     int sm_idle;                     // zeros: the plane of threads without a block
+    int sm_st;                       // copy of st for the gathered stages (indexed by a loop counter there; as kernel parameters: 2 to 4 % of a solve)
     int P;                           // pitch and member stride of the first level's arrays
     long long S;
 };
@@ -544,7 +545,7 @@ __device__ __forceinline__ void sweeps(Ctx<T, S> &c, int k, int from, int pairs,
 template <class T, int b, int S>
 __device__ __forceinline__ void load_cond(const ClusterArgs &a, const Ctx<T, S> &c, int k, Cond<T, b> &q)
 {
-    const ClStageArgs &st = a.st[c.id];
+    const ClStageArgs &st = S > 0 ? sp<const ClStageArgs>(a.sm_st)[c.id] : a.st[0];
     if constexpr (S > 0) q.load(sp<const T>(st.simg[k]) + c.tid, st.nt);
     else if constexpr (sizeof(T) == 4) q.load(sp<const T>(st.simg[k]) + c.kind[k], st.nrec[k]);
     else q.load(reinterpret_cast<const T *>(st.img[k]) + c.kind[k], st.nrec[k]);
@@ -580,12 +581,13 @@ template <class T, int b> __device__ __forceinline__ void prolong(unsigned int m
 // each stage's iterates wait in local memory while the deeper ones run.
 template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a, int tid, int *fail)
 {
+    const ClStageArgs *sst = sp<const ClStageArgs>(a.sm_st);
     T save[CL_STAGES][10];
     Ctx<T, 1> c;
     c.tid = tid; c.rank = 0; c.fail = fail;
     T f[2][2], e[2][2], f1[1][1], e1[1][1];
     auto enter = [&](int s) {
-        const ClStageArgs &st = a.st[s];
+        const ClStageArgs &st = sst[s];
         c.id = s; c.nt = st.nt;
         const bool act = tid < st.bw * st.bh;
         // tid / bw by the stage's reciprocal (exact for tid < 2^16)
@@ -602,12 +604,12 @@ template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a
         return int2{bx, by};
     };
     auto cond1 = [&](Cond<T, 1> &q) {
-        const ClStageArgs &st = a.st[c.id];
+        const ClStageArgs &st = sst[c.id];
         q.load(sp<const T>(st.simg[st.B == 2 ? 1 : 0]) + tid, st.nt);
     };
     int s = 1;
     for (;; ++s) {                                           // down
-        const ClStageArgs &st = a.st[s], &up = a.st[s - 1];
+        const ClStageArgs &st = sst[s], &up = sst[s - 1];
         const int2 xy = enter(s);
         const bool act = (c.flags & CF_ACT) != 0, last = s + 1 == a.nst;
         const int seq = up.seq[up.nlev - 1];
@@ -641,14 +643,14 @@ template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a
         residual<T, 1, 1>(c, 1, q, st.seq[st.nlev - 1], f1, e1, res);
         if (act) *sp<T>(st.rp + (xy.y * st.bw + xy.x) * (int)sizeof(T)) = res[0][0];
         stage_sync<1>(s, st.nt);
-        if (tid >= a.st[s + 1].nt) break;
+        if (tid >= sst[s + 1].nt) break;
         T *sv = save[s];
         sv[0] = f[0][0]; sv[1] = f[0][1]; sv[2] = f[1][0]; sv[3] = f[1][1];
         sv[4] = e[0][0]; sv[5] = e[0][1]; sv[6] = e[1][0]; sv[7] = e[1][1];
         sv[8] = f1[0][0]; sv[9] = e1[0][0];
     }
     for (bool fresh = true; s >= 1; --s, fresh = false) {    // up
-        const ClStageArgs &st = a.st[s];
+        const ClStageArgs &st = sst[s];
         const bool last = s + 1 == a.nst;
         if (!fresh) {
             const T *sv = save[s];
@@ -660,7 +662,7 @@ template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a
         const bool act = (c.flags & CF_ACT) != 0;
         if (!last) {
             stage_sync<1>(s, st.nt);                         // the deeper stages' result is complete
-            const ClStageArgs &nx = a.st[s + 1];
+            const ClStageArgs &nx = sst[s + 1];
             const T ec = *sp<const T>(nx.plane[0] + (((xy.y >> 1) + 1) * nx.pitch[0] + CL_PAD + (xy.x >> 1)) * (int)sizeof(T));
             if (c.fm >> 20 & 1) e1[0][0] += ec;
         }
@@ -1080,6 +1082,8 @@ __global__ void __launch_bounds__(ClLimit<T, B>::threads, 1) k_cluster(const __g
     }
     T *lut = sp<T>(a.sm_lut);
     const T cx = sizeof(T) == 4 ? (T)sa.cxf : (T)sa.cxd, cy = sizeof(T) == 4 ? (T)sa.cyf : (T)sa.cyd;
+    if (rank == 0)
+        for (int q = tid; q < (int)(sizeof(a.st) / 4); q += blockDim.x) sp<int>(a.sm_st)[q] = reinterpret_cast<const int *>(a.st)[q];
     // conductance tables, and the gathered stages' fluid bits
     for (int s = sizeof(T) == 4 ? 0 : 1; s < (rank == 0 ? a.nst : 1); ++s) {
         const ClStageArgs &st = a.st[s];
@@ -1663,6 +1667,7 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
         a.st[s].fo = (int)o;
         if (a.st[s].wide) o = up16(o + sizeof(T) * (size_t)a.st[s].ni);
     }
+    a.sm_st = (int)o; o = up16(o + sizeof(a.st));
     a.sm_lut = (int)o; o = up16(o + 32 * sizeof(T));
     a.sm_red = (int)o; o = up16(o + 32 * 8);
     a.sm_slot = (int)o; o = up16(o + 2 * CL_MAXC * 8);
