@@ -1058,10 +1058,15 @@ __device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<fl
 // ------------------------------------------------------------------------------------ the kernel
 // Threads per block at most: the registers of 640 threads fit twice 48; a mixed 4 x 4 block keeps its
 // iterate and right-hand side (32 values) with one level's conductances (16) in 96 registers.
-template <class T, int B> struct ClLimit { static constexpr int threads = B == 2 ? 768 : sizeof(T) == 4 ? 640 : 352; };
+// FP64 2 x 2 blocks: 152 registers without spills up to 192 threads, with which two blocks still share an SM;
+// beyond, 128 (512 threads), for the same reason.  (At 80 registers and 768 threads 400 bytes per thread spilled: 128 x 64,
+// one member at a time: 50.5 ms, now 42.5 ms; 176 x 80, 17 members: 10.4 ms, with 152 registers and one block per
+// SM 13.7 ms, with 128 registers 9.4 ms.)
+constexpr int CL_FEW_THREADS = 192, CL_FEW_BOUND = 384;
+template <class T, int B> struct ClLimit { static constexpr int threads = B == 2 ? (sizeof(T) == 4 ? 768 : 512) : sizeof(T) == 4 ? 640 : 352; };
 
-template <class T, int B, bool FIRST, bool MULTI>
-__global__ void __launch_bounds__(ClLimit<T, B>::threads, 1) k_cluster(const __grid_constant__ ClusterArgs a, const __grid_constant__ SolveArgs sa)
+template <class T, int B, bool FIRST, bool MULTI, int BOUND>
+__global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ ClusterArgs a, const __grid_constant__ SolveArgs sa)
 {
     __shared__ ClScal<T, decltype(Dot<T>::v)> sc;
     __shared__ int s_fail;
@@ -1713,7 +1718,9 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
 
 template <class T, int B, bool FIRST, bool MULTI> static cudaError_t launch_k(const ClusterPlan &p, const SolveArgs &sa, int M, cudaStream_t st, bool query, int *active)
 {
-    auto kern = k_cluster<T, B, FIRST, MULTI>;
+    auto kern = k_cluster<T, B, FIRST, MULTI, ClLimit<T, B>::threads>;
+    if constexpr (sizeof(T) == 8 && B == 2)
+        if (p.threads <= CL_FEW_THREADS) kern = k_cluster<T, B, FIRST, MULTI, CL_FEW_BOUND>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.a.C * M);
     cfg.blockDim = dim3(p.threads);
