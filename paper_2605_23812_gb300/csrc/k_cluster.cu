@@ -1063,6 +1063,9 @@ __device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<fl
 // one member at a time: 50.5 ms, now 42.5 ms; 176 x 80, 17 members: 10.4 ms, with 152 registers and one block per
 // SM 13.7 ms, with 128 registers 9.4 ms.)
 constexpr int CL_FEW_THREADS = 192, CL_FEW_BOUND = 384;
+// Mixed 4 x 4 blocks up to 512 threads: 128 registers where an SM holds one block anyway (more than 320 threads,
+// or 112 KB; 96 registers spill 460 bytes per thread): 256 x 128, 33 members 7.31 -> 6.56 ms, 5 members 2.96 -> 2.70 ms.
+constexpr int CL_MID_BOUND = 512;
 template <class T, int B> struct ClLimit { static constexpr int threads = B == 2 ? (sizeof(T) == 4 ? 768 : 512) : sizeof(T) == 4 ? 640 : 352; };
 
 template <class T, int B, bool FIRST, bool MULTI, int BOUND>
@@ -1721,6 +1724,8 @@ template <class T, int B, bool FIRST, bool MULTI> static cudaError_t launch_k(co
     auto kern = k_cluster<T, B, FIRST, MULTI, ClLimit<T, B>::threads>;
     if constexpr (sizeof(T) == 8 && B == 2)
         if (p.threads <= CL_FEW_THREADS) kern = k_cluster<T, B, FIRST, MULTI, CL_FEW_BOUND>;
+    if constexpr (sizeof(T) == 4 && B == 4 && FIRST)
+        if (p.threads <= CL_MID_BOUND && (p.threads > 320 || p.smem > 112 * 1024)) kern = k_cluster<T, B, FIRST, MULTI, CL_MID_BOUND>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.a.C * M);
     cfg.blockDim = dim3(p.threads);
