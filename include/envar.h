@@ -294,6 +294,12 @@ int envar_time_kernel(envar_handle h, int which, int reps, double *ms_per_launch
  * solver's work vectors of every member slot. */
 int envar_apply_preconditioner(envar_handle h, const double *r_dev, double *z_dev);
 
+/* Diagnostics of one handle, for tests (a batch that holds the handle keeps what it has captured).
+ * ENVAR_DIAG_WAIT_LIMIT: how often the blocks of a cluster pressure solve try a wait on one another
+ * before they give up and mark the member ENVAR_ST_DIVERGENCE; 0: once, -1: the default. */
+enum { ENVAR_DIAG_WAIT_LIMIT = 0 };
+int envar_set_diagnostic(envar_handle h, int what, int value);
+
 /* Reference gradient by the discrete adjoint (Sec. 3.2, Eq. adjoint_discrete and
  * Eq. gradient_forcing, in their discrete form): the exact gradient of the DOMAIN cost J(f) of one
  * forward run from the handle's initial state, with the steady forcing f on the control cells,

@@ -99,6 +99,7 @@ def lib():
         "envar_kernel_launches": [H, ctypes.POINTER(ctypes.c_longlong)],
         "envar_time_kernel": [H, c_int, c_int, ctypes.POINTER(c_double)],
         "envar_apply_preconditioner": [H, c_void_p, c_void_p],
+        "envar_set_diagnostic": [H, c_int, c_int],
         "envar_adjoint_gradient": [H, c_void_p, c_void_p, c_int, c_void_p],
         "envar_autotune": [H, c_int, ctypes.POINTER(c_double), ctypes.POINTER(c_int)],
         "envar_get_config": [H, ctypes.POINTER(Config)],
@@ -317,6 +318,10 @@ class Ensemble:
         t.cuda.current_stream().synchronize()
         self._check(lib().envar_apply_preconditioner(self._h, _ptr(rr), _ptr(z)), "envar_apply_preconditioner")
         return z
+
+    def set_diagnostic(self, what: int, value: int):
+        """Diagnostics for tests (see envar_set_diagnostic)."""
+        self._check(lib().envar_set_diagnostic(self._h, int(what), int(value)), "envar_set_diagnostic")
 
     def time_kernel(self, which: int, reps: int = 20) -> float:
         ms = c_double()

@@ -1056,6 +1056,7 @@ extern "C" int envar_init(envar_handle *out, const envar_config *cfg, void *cuda
         pc.rtol_abs = c.div_tol * h->g.hxy / h->g.dt;
         pc.cimg = h->d_cimg;
         pc.cimg_bytes = h->cimg_bytes;
+        pc.wait_limit = CLUSTER_WAIT_LIMIT;
         pc.solve = h->plan;
         pc.coarse = h->plan_coarse;
         {
@@ -2323,6 +2324,15 @@ extern "C" int envar_autotune(envar_handle h, int probe_steps, double *best_ms_p
         set_err(h, "envar_autotune: no candidate kept every member within div_tol; parameters unchanged");
         return ENVAR_ESTATE;
     }
+    return ENVAR_OK;
+}
+
+extern "C" int envar_set_diagnostic(envar_handle h, int what, int value)
+{
+    if (!h || what != ENVAR_DIAG_WAIT_LIMIT || value < -1) return ENVAR_EINVAL;
+    h->pc.wait_limit = value < 0 ? CLUSTER_WAIT_LIMIT : value;
+    CK(cudaStreamSynchronize(h->st));
+    drop_graphs(h);
     return ENVAR_OK;
 }
 

@@ -329,6 +329,7 @@ void launch_export_state(const Grid &g, const double *u, const double *v, const 
 // Cluster pressure solve (k_cluster.cu): a member's whole solve, or the V-cycle of the levels below
 // the first, in one thread-block cluster.
 struct ClusterPlan;
+constexpr int CLUSTER_WAIT_LIMIT = 1 << 17;
 struct ClusterHostLevel {           // host copy of a multigrid level, pitch P
     int nx, ny, P;
     const uint8_t *F, *open;        // fluid cells; open-face bits (first level)
@@ -369,6 +370,7 @@ struct PoissonCfg {
     MixConst mc;
     const unsigned char *cimg;      // coarse-block shared-memory image of the coarse levels' constants
     int cimg_bytes;                 // its size (a multiple of 16)
+    int wait_limit;                 // tries of a wait inside the cluster kernels (CLUSTER_WAIT_LIMIT)
     ClusterPlan *solve;             // the whole solve in a cluster per member, or
     ClusterPlan *coarse;            // the V-cycle's levels from 1 on (FP32); nullptr: tiled kernels
 };

@@ -19,14 +19,17 @@
 // uses the operations of the tiled kernels in their order, so FP32 iterates equal theirs bit for bit;
 // dot products are df64 (or FP64) sums in another order.
 //
-// Every wait has an iteration limit; a wait that runs out marks the member unconverged and the
-// kernel ends.
+// Every wait on a barrier in shared memory has an iteration limit.  A thread whose wait ran out sends
+// nothing more to other blocks and waits for nothing more, so the others' waits run out too; all blocks
+// learn of it at the cluster barrier that ends a refinement (agree), leave together and mark the member's
+// status as a solve that did not converge.
 #include <algorithm>
 #include <cstring>
 #include <map>
 #include <utility>
 #include <vector>
 
+#include "../../include/envar.h"
 #include "df64.cuh"
 #include "envar_internal.cuh"
 
@@ -63,17 +66,24 @@ __device__ __forceinline__ bool mb_try(unsigned int bar, unsigned int phase)
                  : "memory");
     return ok != 0;
 }
-constexpr int CL_WAIT_LIMIT = 1 << 17;
-// bounded wait; once one ran out (*fail) later waits return at once
-__device__ __forceinline__ void mb_wait(unsigned int bar, unsigned int phase, int *fail)
+// a block's record of its waits
+struct ClWatch {
+    int failed;                      // one ran out
+    int limit;                       // tries of a wait
+    int any[2];                      // one ran out in some block of the cluster (agree; used in turn)
+};
+// bounded wait, false if it ran out; once one did, the block's other waits return at once
+__device__ __forceinline__ bool mb_wait(unsigned int bar, unsigned int phase, ClWatch *w)
 {
-    if (mb_try(bar, phase)) return;
-    volatile int *vf = fail;
+    if (mb_try(bar, phase)) return true;
+    volatile ClWatch *v = w;
 #pragma unroll 1
-    for (int k = 0; k < CL_WAIT_LIMIT && !*vf; ++k)
-        if (mb_try(bar, phase)) return;
-    *vf = 1;
+    for (int k = v->limit; k > 0 && !v->failed; --k)
+        if (mb_try(bar, phase)) return true;
+    v->failed = 1;
+    return false;
 }
+__device__ __forceinline__ bool has_failed(const ClWatch *w) { return *(const volatile int *)&w->failed != 0; }
 __device__ __forceinline__ void cluster_sync_all()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -162,6 +172,7 @@ struct ClusterArgs {
 };
 struct SolveArgs {                   // one pressure solve (mode 0) or one V-cycle of the levels from la (mode 1)
     int mode, max_outer, first_o, one, count_last, max_inner, inner_guard;   // one: a single refinement (from first_o)
+    int wait_limit;                  // tries of a wait in the kernel
     double inner_rtol2, rtol_abs;
     MixConst mc;
     double cxd, cyd;
@@ -199,7 +210,7 @@ template <class T, int S> struct Ctx {
     unsigned int pushS[3], pushN[3], rbarS, rbarN;
     int rxS, rxN;
     int n, gat, nred;
-    int *fail;
+    ClWatch *watch;
 };
 // barriers (byte offsets): halo south [2], halo north [2], reductions [2], gather, gathered result
 enum { BAR_S = 0, BAR_N = 16, BAR_RED = 32, BAR_GAT = 48, BAR_RES = 56 };
@@ -277,6 +288,8 @@ __device__ __forceinline__ void exchange(Ctx<T, S> &c, int k, const T (&e)[b][b]
 {
     // (threads without a block keep zeros in a plane of their own: no branch)
     const int o = c.own[k], p = c.pitch[k];
+    bool dead = false;
+    if constexpr (S == 0 && MULTI) dead = has_failed(c.watch);
     if constexpr (S == 0 && MULTI) {
         const unsigned int off = 8u * (c.n & 1);
         if (c.flags & (CF_PUSH_S | CF_PUSH_N)) {
@@ -294,14 +307,18 @@ __device__ __forceinline__ void exchange(Ctx<T, S> &c, int k, const T (&e)[b][b]
     }
     if constexpr (S == 0 && MULTI) {
         const unsigned int off = 8u * (c.n & 1), ph = (c.n >> 1) & 1;
-        if (c.tid == 0) {
+        // (a barrier whose bytes did not come is not armed a second time: the block's waits of the exchange
+        // before last, which used this one, ended ahead of the last exchange's __syncthreads)
+        if (c.tid == 0 && !dead) {
             if (c.rxS) mb_expect(sa32(BAR_S) + off, c.rxS * b * (int)sizeof(T));
             if (c.rxN) mb_expect(sa32(BAR_N) + off, c.rxN * b * (int)sizeof(T));
         }
         __syncthreads();
         if (c.flags & (CF_WAIT_S | CF_WAIT_N)) {
-            if (c.flags & CF_WAIT_S) mb_wait(sa32(BAR_S) + off, ph, c.fail);
-            if (c.flags & CF_WAIT_N) mb_wait(sa32(BAR_N) + off, ph, c.fail);
+            bool ok = true;
+            if (c.flags & CF_WAIT_S) ok = mb_wait(sa32(BAR_S) + off, ph, c.watch);
+            if (c.flags & CF_WAIT_N) ok = mb_wait(sa32(BAR_N) + off, ph, c.watch) && ok;
+            if (!ok) c.flags &= ~(CF_PUSH_S | CF_PUSH_N | CF_WAIT_S | CF_WAIT_N);
         }
         c.n++;
         __syncwarp();
@@ -579,12 +596,12 @@ template <class T, int b> __device__ __forceinline__ void prolong(unsigned int m
 // result.  One copy of the code runs every stage (the instructions of a V-cycle have to stay in the
 // instruction cache: with a copy per stage the whole kernel was 420 KB and ran at half the speed);
 // each stage's iterates wait in local memory while the deeper ones run.
-template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a, int tid, int *fail)
+template <class T> __device__ __forceinline__ void gathered(const ClusterArgs &a, int tid)
 {
     const ClStageArgs *sst = sp<const ClStageArgs>(a.sm_st);
     T save[CL_STAGES][10];
     Ctx<T, 1> c;
-    c.tid = tid; c.rank = 0; c.fail = fail;
+    c.tid = tid; c.rank = 0;
     T f[2][2], e[2][2], f1[1][1], e1[1][1];
     auto enter = [&](int s) {
         const ClStageArgs &st = sst[s];
@@ -723,10 +740,10 @@ template <class T> __device__ __forceinline__ void gathered_wide(const ClusterAr
     for (int h = 0; h < 2 * a.coarse_sweeps; ++h) half(h & 1, h == 0);
     for (int h = 0; h < 2 * a.coarse_sweeps; ++h) half((h & 1) ^ 1, false);
 }
-template <class T> __device__ __forceinline__ void gathered_any(const ClusterArgs &a, int tid, int *fail)
+template <class T> __device__ __forceinline__ void gathered_any(const ClusterArgs &a, int tid)
 {
     if (sizeof(T) == 4 && a.st[1].wide) gathered_wide<T>(a, tid);
-    else gathered<T>(a, tid, fail);
+    else gathered<T>(a, tid);
 }
 
 // hand the residual of the cluster's last level to the gathered stages and return the coarse
@@ -742,27 +759,32 @@ template <class T, bool MULTI> __device__ __forceinline__ T gather_stage(const C
     if constexpr (MULTI) {
         const unsigned int gbar = sa32(BAR_GAT), rbar = sa32(BAR_RES);
         const unsigned int ph = c.gat & 1;
-        if (c.rank == 0 && c.tid == 0) mb_expect(gbar, a.nact * (int)sizeof(T));
-        if (act) st_async(remote(sa32(at), 0), res, remote(gbar, 0));
+        // (a thread whose own wait ran out sees the mark here; others send one gather more at most, as they
+        // wait for its result)
+        const bool live = !has_failed(c.watch);
+        if (live) {
+            if (c.rank == 0 && c.tid == 0) mb_expect(gbar, a.nact * (int)sizeof(T));
+            if (act) st_async(remote(sa32(at), 0), res, remote(gbar, 0));
+        }
         if (c.rank == 0 && c.tid < nx.nt) {
-            mb_wait(gbar, ph, c.fail);
+            const bool ok = live && mb_wait(gbar, ph, c.watch);
             __syncwarp();
-            gathered_any<T>(a, c.tid, c.fail);
+            gathered_any<T>(a, c.tid);
             stage_sync<1>(1, nx.nt);
-            if (c.tid < a.C) {
+            if (c.tid < a.C && ok) {
                 asm volatile("fence.acq_rel.cluster;" ::: "memory");
                 mb_arrive_remote(remote(rbar, c.tid));
             }
             __syncwarp();
         }
-        mb_wait(rbar, ph, c.fail);
+        if (live) mb_wait(rbar, ph, c.watch);
         c.gat++;
         __syncwarp();
         return act ? ld_remote(remote(sa32(from), 0), (T)0) : (T)0;
     } else {
         if (act) *sp<T>(at) = res;
         __syncthreads();
-        if (c.tid < nx.nt) gathered_any<T>(a, c.tid, c.fail);
+        if (c.tid < nx.nt) gathered_any<T>(a, c.tid);
         __syncthreads();
         return act ? *sp<const T>(from) : (T)0;
     }
@@ -827,9 +849,11 @@ __device__ __forceinline__ V cluster_total(const ClusterArgs &a, Ctx<T, 0> &c, V
             const int par = c.nred & 1;
             const unsigned int bar = sa32(BAR_RED) + 8u * par;
             const unsigned int slots = sa32(a.sm_slot) + 8u * (CL_MAXC * par);
-            if (lane == 0) mb_expect(bar, a.C * 8);
-            if (lane < a.C) st_async(remote(slots + 8u * c.rank, lane), as_bits(tot), remote(bar, lane));
-            mb_wait(bar, (c.nred >> 1) & 1, c.fail);
+            if (!has_failed(c.watch)) {                      // (the same for the warp: no wait of the block is under way)
+                if (lane == 0) mb_expect(bar, a.C * 8);
+                if (lane < a.C) st_async(remote(slots + 8u * c.rank, lane), as_bits(tot), remote(bar, lane));
+                mb_wait(bar, (c.nred >> 1) & 1, c.watch);
+            }
             __syncwarp();
             V y{};
             if (lane < a.C) y = as_acc(sp<const double>(a.sm_slot)[CL_MAXC * par + lane], V{});
@@ -838,6 +862,20 @@ __device__ __forceinline__ V cluster_total(const ClusterArgs &a, Ctx<T, 0> &c, V
     }
     c.nred++;
     return tot;
+}
+
+// Cluster barrier at which every block learns whether a wait ran out in any.  Blocks may disagree on
+// whether the solve goes on only after such a wait, and its block has said so here by then: all take
+// part in the same barriers, and none leaves while others may reach its shared memory.  turn alternates.
+template <bool MULTI> __device__ __forceinline__ bool agree(const ClusterArgs &a, ClWatch *w, int tid, int turn)
+{
+    __syncthreads();                                         // the block's waits are over
+    if constexpr (!MULTI) return false;
+    if (tid < a.C && has_failed(w))
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(sptr(&w->any[turn]), tid)), "r"(1) : "memory");
+    __syncwarp();
+    cluster_sync_all();
+    return *(volatile int *)&w->any[turn] != 0;
 }
 
 // shared scalars of the solve, written by thread 0 (V: f2 or double)
@@ -995,7 +1033,7 @@ __device__ __forceinline__ double outer_res(const ClusterArgs &a, const SolveArg
 // gives enters the pressure and the next guess, and cancels almost to zero, so its bits depend on the
 // order; mixed handles take the same bits on either solve path.
 template <bool MULTI>
-__device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<float, 0> &c, long long off)
+__device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<float, 0> &c, long long off, int turn, bool *failed)
 {
     const int gx = (sa.nx + 63) / 64, gy = (sa.ny + 31) / 32, nb = gx * gy;
     const int lane = c.tid & 31, w = c.tid >> 5, nw = (int)blockDim.x >> 5;
@@ -1040,8 +1078,7 @@ __device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<fl
         v = warp_sum_df(v);
         if (lane == 0) *reinterpret_cast<float2 *>(slots + c.rank + t * a.C) = make_float2(v.h, v.l);
     }
-    if constexpr (MULTI) cluster_sync_all();
-    else __syncthreads();
+    *failed = agree<MULTI>(a, c.watch, c.tid, turn);
     double tot = 0.0;
     if (c.rank == 0 && w == 0) {
         f2 xs{0.f, 0.f};
@@ -1072,14 +1109,14 @@ template <class T, int B, bool FIRST, bool MULTI, int BOUND>
 __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ ClusterArgs a, const __grid_constant__ SolveArgs sa)
 {
     __shared__ ClScal<T, decltype(Dot<T>::v)> sc;
-    __shared__ int s_fail;
+    __shared__ ClWatch watch;
     const int rank = MULTI ? cluster_rank() : 0;
     const int m = blockIdx.x / a.C, tid = threadIdx.x;
     if (sa.ctl[m].outer_done) return;                        // every block of the cluster reads the same word
     if (sa.mode == 1 && sa.inner_guard && sa.ctl[m].inner_done) return;
     const long long off = (long long)m * a.S;
     if (tid == 0) {
-        s_fail = 0;
+        watch = ClWatch{0, sa.wait_limit, {0, 0}};
         for (int q = 0; q < 8; ++q) mb_init(sa32(8 * q), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1109,7 +1146,7 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
         lut[16 + q] = (d != (T)0) ? (T)1 / d : (T)0;
     }
     Ctx<T, 0> c;
-    c.tid = tid; c.rank = rank; c.id = 0; c.nt = a.nt; c.fail = &s_fail;
+    c.tid = tid; c.rank = rank; c.id = 0; c.nt = a.nt; c.watch = &watch;
     c.n = c.gat = c.nred = 0;
     const int4 rec = a.rec[rank * a.nt + tid];
     const int bx = rec.x & 0xffff, by = (rec.x >> 16) & 0xffff;
@@ -1152,6 +1189,7 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
 
     const long long at = off + (long long)by * B * a.P + bx * B;   // the block's first cell
     T f[B][B], e[B][B];
+    bool failed = false;
 
     if constexpr (!FIRST) {
         // mode 1: one V-cycle of the levels from la
@@ -1166,6 +1204,7 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
 #pragma unroll
             for (int r = 0; r < B; ++r) st_row(reinterpret_cast<T *>(sa.e) + at + (long long)r * a.P, e[r]);
         }
+        failed = agree<MULTI>(a, &watch, tid, 0);
     } else {
         Open<T, B> q;
         q.cx = cx; q.cy = cy; q.lut = lut;
@@ -1182,7 +1221,8 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
         bool done = false;
         bool closed = false;                                 // the loop ended at a residual
         double rmax_d = 0.0;
-        for (int o = sa.first_o;; ++o) {
+        int o = sa.first_o;
+        for (;; ++o) {
             {
                 const auto rm = outer_res<B>(a, sa, c, off, bx, by, q.lo, q.hi, fl, f);
                 const double t = cluster_total<T, double, MULTI, true>(a, c, (double)rm);
@@ -1350,15 +1390,14 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
                     have_acc = true;
                 }
             }
-            if constexpr (MULTI) cluster_sync_all();         // x of every block before the next residual reads it
-            else __syncthreads();
-            if (sa.one) break;
+            failed = agree<MULTI>(a, &watch, tid, o & 1);    // x of every block before the next residual reads it
+            if (failed || sa.one) break;
         }
         // totals and flags of the member (the fluid sum of x is its mean's numerator)
         double xs = 0.0;
         if (!closed) {
         } else if constexpr (sizeof(T) == 4) {
-            xs = fluid_sum_mx<MULTI>(a, sa, c, off);
+            xs = fluid_sum_mx<MULTI>(a, sa, c, off, o & 1, &failed);
         } else {
             double v = 0.0;
             if (act) {
@@ -1372,21 +1411,30 @@ __global__ void __launch_bounds__(BOUND, 1) k_cluster(const __grid_constant__ Cl
                 }
             }
             xs = cluster_total<T, double, MULTI, false>(a, c, v);
+            failed = agree<MULTI>(a, &watch, tid, o & 1);
         }
         if (rank == 0 && tid == 0) {
             MemberRed &red = sa.rc.red[m];
-            if (closed) {
-                red.val[RS_RMAX] = s_fail ? 1e300 : rmax_d;  // a wait ran out: the member counts as unconverged
-                red.val[RS_XSUM] = xs;
+            if (closed || failed) {
+                red.val[RS_RMAX] = failed ? 1e300 : rmax_d;
+                red.val[RS_XSUM] = failed ? 0.0 : xs;
             }
             MemberCtl &mc = sa.ctl[m];
-            mc.outer_done = done;
-            mc.inner_done = done;
+            mc.outer_done = done && !failed;
+            mc.inner_done = done && !failed;
             mc.outer_its += outer_its;
             mc.inner_its += inner_its;
         }
     }
-    if constexpr (MULTI) cluster_sync_all();                 // no block leaves while others may reach its shared memory
+    if (failed) {
+        // a wait ran out: the member counts as unconverged.  Stores that nobody waited for may still be on
+        // their way; no block sends more, and a tenth of a millisecond is two hundred times their latency.
+        if (rank == 0 && tid == 0) atomicOr(&sa.ctl[m].status, ENVAR_ST_DIVERGENCE);
+#pragma unroll 1
+        for (int k = 0; k < 16; ++k) __nanosleep(8000);
+        cluster_sync_all();
+    }
+    // (otherwise the last agree ended all access to other blocks' shared memory: no barrier before the exit)
 }
 
 // ------------------------------------------------------------------------------------ plan (host)
@@ -1818,6 +1866,7 @@ void launch_cluster_solve(const Grid &g, const Level &L0, int M, const PoissonBu
     set_sweeps(p, pc);
     SolveArgs sa{};
     sa.mode = 0;
+    sa.wait_limit = pc.wait_limit;
     sa.max_outer = pc.max_outer; sa.max_inner = pc.max_inner;
     sa.inner_rtol2 = pc.inner_rtol2; sa.rtol_abs = pc.rtol_abs;
     sa.mc = pc.mc;
@@ -1849,6 +1898,7 @@ void launch_cluster_vcycle(int M, const float *f, float *e, const PoissonCfg &pc
     SolveArgs sa{};
     sa.mode = 1;
     sa.inner_guard = inner_guard;
+    sa.wait_limit = pc.wait_limit;
     sa.f = f; sa.e = e;
     sa.ctl = ctl;
     if (dispatch<float>(*p, sa, M, st, false, nullptr) != cudaSuccess) note_capture_failure();
