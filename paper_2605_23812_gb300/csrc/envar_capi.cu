@@ -1991,9 +1991,12 @@ extern "C" int envar_apply_preconditioner(envar_handle h, const double *r_dev, d
         launch_vcycle<double>(h->g, h->lev, h->Mall, h->pb, h->pc, h->pt, h->d_ctl, h->st);
         launch_cells_out<double>(h->g, (const double *)h->pb.z, z_dev, h->st);
     }
-    // r_dev may be nonzero in solid cells: the solves count on zeros there
+    // r_dev may be nonzero in solid cells, and not finite: then the first slot's iterates (z, and the guess of
+    // the pre-smoothing) are not finite in solid cells either.  The solves count on zeros there.
     CK(cudaMemsetAsync(h->pb.r, 0, tsz * (size_t)h->g.S * h->Mall, h->st));
     CK(cudaMemsetAsync(h->pb.lev_f[1], 0, tsz * (size_t)h->lev[1].S * h->Mall, h->st));
+    CK(cudaMemsetAsync(h->pb.z, 0, tsz * (size_t)h->g.S, h->st));
+    CK(cudaMemsetAsync(h->pb.lev_t[0], 0, tsz * (size_t)h->lev[0].S, h->st));
     CK(cudaStreamSynchronize(h->st));
     CK(cudaGetLastError());
     return ENVAR_OK;
