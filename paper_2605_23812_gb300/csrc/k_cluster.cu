@@ -72,16 +72,20 @@ struct ClWatch {
     int limit;                       // tries of a wait
     int any[2];                      // one ran out in some block of the cluster (agree; used in turn)
 };
-// bounded wait, false if it ran out; once one did, the block's other waits return at once
-__device__ __forceinline__ bool mb_wait(unsigned int bar, unsigned int phase, ClWatch *w)
+// per-thread flags
+enum { CF_WLANE = 1, CF_ELANE = 2, CF_PUSH_S = 4, CF_PUSH_N = 8, CF_WAIT_S = 16, CF_WAIT_N = 32, CF_ACT = 64, CF_PAR = 128,
+       CF_LOST = 256 };              // a wait of this thread ran out
+// bounded wait; once one ran out, the block's other waits return at once.  A thread whose wait ran out
+// neither sends to other blocks nor waits again.  (All of it behind the first try, which nearly always holds.)
+__device__ __forceinline__ void mb_wait(unsigned int bar, unsigned int phase, ClWatch *w, int &flags)
 {
-    if (mb_try(bar, phase)) return true;
+    if (mb_try(bar, phase)) return;
     volatile ClWatch *v = w;
 #pragma unroll 1
     for (int k = v->limit; k > 0 && !v->failed; --k)
-        if (mb_try(bar, phase)) return true;
+        if (mb_try(bar, phase)) return;
     v->failed = 1;
-    return false;
+    flags = (flags & ~(CF_PUSH_S | CF_PUSH_N | CF_WAIT_S | CF_WAIT_N)) | CF_LOST;
 }
 __device__ __forceinline__ bool has_failed(const ClWatch *w) { return *(const volatile int *)&w->failed != 0; }
 __device__ __forceinline__ void cluster_sync_all()
@@ -132,8 +136,6 @@ __device__ __forceinline__ double ld_remote(unsigned int a, double)
 constexpr int CL_MAXC = 16;          // blocks per cluster at most
 constexpr int CL_STAGES = 4;         // the cluster's levels, then up to three gathered stages
 constexpr int CL_PAD = 4;            // columns left of a plane's cells (alignment of vector accesses)
-// per-thread flags
-enum { CF_WLANE = 1, CF_ELANE = 2, CF_PUSH_S = 4, CF_PUSH_N = 8, CF_WAIT_S = 16, CF_WAIT_N = 32, CF_ACT = 64, CF_PAR = 128 };
 
 struct ClSlab { int cb0, rb0, wb, hb, rxS, rxN; };   // block columns / rows held, blocks pushed in from south / north
 struct ClStageArgs {
@@ -315,10 +317,8 @@ __device__ __forceinline__ void exchange(Ctx<T, S> &c, int k, const T (&e)[b][b]
         }
         __syncthreads();
         if (c.flags & (CF_WAIT_S | CF_WAIT_N)) {
-            bool ok = true;
-            if (c.flags & CF_WAIT_S) ok = mb_wait(sa32(BAR_S) + off, ph, c.watch);
-            if (c.flags & CF_WAIT_N) ok = mb_wait(sa32(BAR_N) + off, ph, c.watch) && ok;
-            if (!ok) c.flags &= ~(CF_PUSH_S | CF_PUSH_N | CF_WAIT_S | CF_WAIT_N);
+            if (c.flags & CF_WAIT_S) mb_wait(sa32(BAR_S) + off, ph, c.watch, c.flags);
+            if (c.flags & CF_WAIT_N) mb_wait(sa32(BAR_N) + off, ph, c.watch, c.flags);
         }
         c.n++;
         __syncwarp();
@@ -759,25 +759,23 @@ template <class T, bool MULTI> __device__ __forceinline__ T gather_stage(const C
     if constexpr (MULTI) {
         const unsigned int gbar = sa32(BAR_GAT), rbar = sa32(BAR_RES);
         const unsigned int ph = c.gat & 1;
-        // (a thread whose own wait ran out sees the mark here; others send one gather more at most, as they
-        // wait for its result)
-        const bool live = !has_failed(c.watch);
-        if (live) {
+        // (threads whose own waits were met send one gather more at most, as they wait for its result)
+        if (!(c.flags & CF_LOST)) {
             if (c.rank == 0 && c.tid == 0) mb_expect(gbar, a.nact * (int)sizeof(T));
             if (act) st_async(remote(sa32(at), 0), res, remote(gbar, 0));
         }
         if (c.rank == 0 && c.tid < nx.nt) {
-            const bool ok = live && mb_wait(gbar, ph, c.watch);
+            if (!(c.flags & CF_LOST)) mb_wait(gbar, ph, c.watch, c.flags);
             __syncwarp();
             gathered_any<T>(a, c.tid);
             stage_sync<1>(1, nx.nt);
-            if (c.tid < a.C && ok) {
+            if (c.tid < a.C && !(c.flags & CF_LOST)) {
                 asm volatile("fence.acq_rel.cluster;" ::: "memory");
                 mb_arrive_remote(remote(rbar, c.tid));
             }
             __syncwarp();
         }
-        if (live) mb_wait(rbar, ph, c.watch);
+        if (!(c.flags & CF_LOST)) mb_wait(rbar, ph, c.watch, c.flags);
         c.gat++;
         __syncwarp();
         return act ? ld_remote(remote(sa32(from), 0), (T)0) : (T)0;
@@ -849,10 +847,10 @@ __device__ __forceinline__ V cluster_total(const ClusterArgs &a, Ctx<T, 0> &c, V
             const int par = c.nred & 1;
             const unsigned int bar = sa32(BAR_RED) + 8u * par;
             const unsigned int slots = sa32(a.sm_slot) + 8u * (CL_MAXC * par);
-            if (!has_failed(c.watch)) {                      // (the same for the warp: no wait of the block is under way)
+            if (!(c.flags & CF_LOST)) {
                 if (lane == 0) mb_expect(bar, a.C * 8);
                 if (lane < a.C) st_async(remote(slots + 8u * c.rank, lane), as_bits(tot), remote(bar, lane));
-                mb_wait(bar, (c.nred >> 1) & 1, c.watch);
+                mb_wait(bar, (c.nred >> 1) & 1, c.watch, c.flags);
             }
             __syncwarp();
             V y{};
