@@ -296,8 +296,10 @@ int envar_apply_preconditioner(envar_handle h, const double *r_dev, double *z_de
 
 /* Diagnostics of one handle, for tests (a batch that holds the handle keeps what it has captured).
  * ENVAR_DIAG_WAIT_LIMIT: how often the blocks of a cluster pressure solve try a wait on one another
- * before they give up and mark the member ENVAR_ST_DIVERGENCE; 0: once, -1: the default. */
-enum { ENVAR_DIAG_WAIT_LIMIT = 0 };
+ * before they give up and mark the member ENVAR_ST_DIVERGENCE; 0: once, -1: the default.
+ * ENVAR_DIAG_TILED_SOLVE: 1: the pressure solve by the tiled kernels on every grid; 0 (the default): in a
+ * thread-block cluster where the grid fits one. */
+enum { ENVAR_DIAG_WAIT_LIMIT = 0, ENVAR_DIAG_TILED_SOLVE = 1 };
 int envar_set_diagnostic(envar_handle h, int what, int value);
 
 /* Reference gradient by the discrete adjoint (Sec. 3.2, Eq. adjoint_discrete and

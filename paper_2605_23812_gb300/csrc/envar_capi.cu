@@ -2332,9 +2332,14 @@ extern "C" int envar_autotune(envar_handle h, int probe_steps, double *best_ms_p
 
 extern "C" int envar_set_diagnostic(envar_handle h, int what, int value)
 {
-    if (!h || what != ENVAR_DIAG_WAIT_LIMIT || value < -1) return ENVAR_EINVAL;
-    h->pc.wait_limit = value < 0 ? CLUSTER_WAIT_LIMIT : value;
+    if (!h || value < -1 || what < 0 || what > ENVAR_DIAG_TILED_SOLVE || (what == ENVAR_DIAG_TILED_SOLVE && value != 0 && value != 1)) return ENVAR_EINVAL;
     CK(cudaStreamSynchronize(h->st));
+    if (what == ENVAR_DIAG_WAIT_LIMIT) {
+        h->pc.wait_limit = value < 0 ? CLUSTER_WAIT_LIMIT : value;
+    } else {
+        h->pc.solve = value ? nullptr : h->plan;
+        h->pc.coarse = value ? nullptr : h->plan_coarse;
+    }
     drop_graphs(h);
     return ENVAR_OK;
 }
