@@ -1526,6 +1526,10 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
     if (la + nloc >= nlev) return nullptr;                   // the coarsest level is in a gathered stage
     const ClusterHostLevel &L = hl[la];
     if (L.nx % B || L.ny % B || bw > 32767 || bh > 32767) return nullptr;
+    // No kernel for these two: a level 1 that one block could hold belongs to a grid that runs whole in a cluster, and FP64
+    // grids of one block run on 2 x 2 blocks of cells (no grid from 16 x 16 to 1400 x 900 in steps of 16, in four boxes, gets here
+    // otherwise).
+    if (C == 1 && (la > 0 || (sizeof(T) == 8 && B == 4))) return nullptr;
     const std::vector<int> &cnt = bl.cnt, &x0 = bl.x0, &x1 = bl.x1;
     const int nact = bl.nact, limit = B == 4 ? ClLimit<T, 4>::threads : ClLimit<T, 2>::threads;
     std::vector<int> first;
@@ -1797,12 +1801,10 @@ template <class T> static cudaError_t dispatch(const ClusterPlan &p, const Solve
 {
     const bool first = p.a.la == 0;
     if constexpr (sizeof(T) == 4) {
-        if (p.a.st[0].B == 4) {
-            if (first) return p.multi ? launch_k<T, 4, true, true>(p, sa, M, st, query, active) : launch_k<T, 4, true, false>(p, sa, M, st, query, active);
-            return p.multi ? launch_k<T, 4, false, true>(p, sa, M, st, query, active) : launch_k<T, 4, false, false>(p, sa, M, st, query, active);
-        }
+        if (!first) return launch_k<T, 4, false, true>(p, sa, M, st, query, active);
+        if (p.a.st[0].B == 4 && !p.multi) return launch_k<T, 4, true, false>(p, sa, M, st, query, active);
     }
-    if (p.a.st[0].B == 4) return p.multi ? launch_k<T, 4, true, true>(p, sa, M, st, query, active) : launch_k<T, 4, true, false>(p, sa, M, st, query, active);
+    if (p.a.st[0].B == 4) return launch_k<T, 4, true, true>(p, sa, M, st, query, active);
     return p.multi ? launch_k<T, 2, true, true>(p, sa, M, st, query, active) : launch_k<T, 2, true, false>(p, sa, M, st, query, active);
 }
 
