@@ -1517,8 +1517,10 @@ struct ClBlocks {
     bool operator()(int x, int y) const { return x >= 0 && y >= 0 && x < bw && y < bh && act[(size_t)y * bw + x]; }
 };
 
-// Build the plan for the levels from la with B x B blocks on C thread blocks.  Returns a device
-// allocation list through `alloc`; nullptr when the grid does not fit the scheme.
+template <class T> static cudaError_t dispatch(const ClusterPlan &p, const SolveArgs &sa, int M, cudaStream_t st, bool query, int *active);
+
+// Build the plan for the levels from la with B x B blocks on C thread blocks, its tables uploaded through `alloc`
+// once nothing else can fail; nullptr when the grid does not fit the scheme or no such cluster is resident.
 template <class T>
 static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, int la, const ClBlocks &bl, int C, const ClusterAlloc &alloc)
 {
@@ -1737,6 +1739,11 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
     P->smem = o;
     P->threads = nt;
     if (o > 226 * 1024) return fail();
+    int resident = 0;
+    if (dispatch<T>(*P, SolveArgs{}, 1, alloc.st, true, &resident) != cudaSuccess || resident < 1) {
+        cudaGetLastError();
+        return fail();
+    }
     // ---- one upload
     std::vector<unsigned char> blob;
     std::vector<std::pair<const void **, size_t>> at;        // pointers and their places in it
@@ -1838,13 +1845,7 @@ ClusterPlan *cluster_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, boo
     for (const Cand &q : cand) {
         const ClBlocks &bl = q.B == 2 ? b2 : b4;
         ClusterPlan *p = mixed ? make_plan<float>(hl, nlev, ncoarse, la, bl, q.C, alloc) : make_plan<double>(hl, nlev, ncoarse, la, bl, q.C, alloc);
-        if (!p) continue;
-        int active = 0;
-        SolveArgs sa{};
-        const cudaError_t e = mixed ? dispatch<float>(*p, sa, 1, alloc.st, true, &active) : dispatch<double>(*p, sa, 1, alloc.st, true, &active);
-        if (e == cudaSuccess && active > 0) return p;
-        cudaGetLastError();
-        delete p;
+        if (p) return p;
     }
     return nullptr;
 }
