@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -1503,12 +1504,19 @@ struct ClBlocks {
     {
         act.assign((size_t)bw * bh, 0);
         cnt.assign(bh, 0); x0.assign(bh, 1 << 30); x1.assign(bh, -1);
-        for (int j = 0; j < bh * B; ++j)
-            for (int x = 0; x < bw; ++x) {
-                unsigned int q = 0;                          // the block's cells of the row (a byte each)
-                std::memcpy(&q, L.F + (size_t)j * L.P + x * B, B);
-                act[(size_t)(j / B) * bw + x] |= q != 0;
+        // the block's cells of a row are a word (a copy of known size: 512 x 256, both B, 0.69 -> 0.05 ms)
+        auto mark = [&](auto word) {
+            for (int j = 0; j < bh * B; ++j) {
+                const uint8_t *f = L.F + (size_t)j * L.P;
+                uint8_t *q = &act[(size_t)(j / B) * bw];
+                for (int x = 0; x < bw; ++x) {
+                    std::memcpy(&word, f + x * sizeof(word), sizeof(word));
+                    q[x] |= word != 0;
+                }
             }
+        };
+        if (B == 4) mark((uint32_t)0);
+        else mark((uint16_t)0);
         for (int y = 0; y < bh; ++y)
             for (int x = 0; x < bw; ++x)
                 if (act[(size_t)y * bw + x]) { ++cnt[y]; x0[y] = std::min(x0[y], x); x1[y] = x; }
@@ -1614,17 +1622,14 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
             if (k > 0 && y == s.rb0 && active(x, y - 1)) fg |= CF_PUSH_S | CF_WAIT_S;
             if (k + 1 < C && y == s.rb0 + s.hb - 1 && active(x, y + 1)) fg |= CF_PUSH_N | CF_WAIT_N;
             if ((x ^ y) & 1) fg |= CF_PAR;
-            unsigned int fl = 0, ob[2] = {0, 0};
-            for (int r = 0; r < B; ++r)
-                for (int i = 0; i < B; ++i) {
-                    const size_t cc = (size_t)(y * B + r) * L.P + x * B + i;
-                    fl |= (L.F[cc] ? 1u : 0u) << (r * B + i);
-                    if (la == 0) {
-                        const int sh = 4 * (r * B + i);
-                        ob[sh >> 5] |= (unsigned int)(L.open[cc] & 15) << (sh & 31);
-                    }
-                }
-            rec[(size_t)k * nt + t] = int4{x | (y << 16), fg | (int)(fl << 16), (int)ob[0], (int)ob[1]};
+            unsigned int fl = 0;
+            uint64_t ob = 0;
+            for (int r = 0; r < B; ++r) {
+                const size_t cc = (size_t)(y * B + r) * L.P + x * B;
+                for (int i = 0; i < B; ++i) fl |= (L.F[cc + i] ? 1u : 0u) << (r * B + i);
+                for (int i = 0; i < B && la == 0; ++i) ob |= (uint64_t)(L.open[cc + i] & 15) << (4 * (r * B + i));
+            }
+            rec[(size_t)k * nt + t] = int4{x | (y << 16), fg | (int)(fl << 16), (int)(unsigned int)ob, (int)(unsigned int)(ob >> 32)};
         }
     }
     // ---- per-level conductances, smoothing factors (their denominators, here) and fluid bits
@@ -1651,39 +1656,55 @@ static ClusterPlan *make_plan(const ClusterHostLevel *hl, int nlev, int ncoarse,
                 continue;
             }
             const int nc = 2 * b * (b + 1), nv = b * b, sh = b == 4 ? 0 : b == 2 ? 16 : 20;
-            std::vector<T> im((size_t)(nc + nv) * n, (T)0);
-            for (int t = 0; t < n; ++t) {
-                int x, y;
-                if (!block(t, &x, &y)) continue;
-                size_t w = t;
+            // the values of block (x, y), and its fluid bits
+            auto record_b = [&](auto size, int x, int y, T *w, size_t stride) {
+                constexpr int b = decltype(size)::value;     // (known when compiled: half the time)
+                int bits = 0;
+                const size_t at = (size_t)(y * b) * H.P + x * b;
                 for (int r = 0; r < b; ++r)
-                    for (int i = 0; i <= b; ++i, w += n) im[w] = (T)H.cw[(size_t)(y * b + r) * H.P + x * b + i];
+                    for (int i = 0; i <= b; ++i, w += stride) *w = (T)H.cw[at + r * H.P + i];
                 for (int r = 0; r <= b; ++r)
-                    for (int i = 0; i < b; ++i, w += n) im[w] = (T)H.cs[(size_t)(y * b + r) * H.P + x * b + i];
+                    for (int i = 0; i < b; ++i, w += stride) *w = (T)H.cs[at + r * H.P + i];
                 for (int r = 0; r < b; ++r)
-                    for (int i = 0; i < b; ++i, w += n) {
-                        const size_t cc = (size_t)(y * b + r) * H.P + x * b + i;
-                        im[w] = (((T)H.cw[cc] + (T)H.cw[cc + 1]) + (T)H.cs[cc]) + (T)H.cs[cc + H.P];
-                        fm[s][t] |= (H.F[cc] ? 1 : 0) << (sh + r * b + i);
+                    for (int i = 0; i < b; ++i, w += stride) {
+                        const size_t cc = at + r * H.P + i;
+                        *w = (((T)H.cw[cc] + (T)H.cw[cc + 1]) + (T)H.cs[cc]) + (T)H.cs[cc + H.P];
+                        bits |= (H.F[cc] ? 1 : 0) << (sh + r * b + i);
                     }
-            }
+                return bits;
+            };
+            auto record = [&](int x, int y, T *w, size_t stride) {
+                return b == 4 ? record_b(std::integral_constant<int, 4>(), x, y, w, stride)
+                     : b == 2 ? record_b(std::integral_constant<int, 2>(), x, y, w, stride)
+                              : record_b(std::integral_constant<int, 1>(), x, y, w, stride);
+            };
+            std::vector<T> im;
             size_t nr = n;
-            if (s == 0) {                                    // merge equal records
+            if (s == 0) {                                    // equal records are one
                 std::map<std::vector<T>, int> seen;
-                std::vector<T> r((size_t)nc + nv);
+                std::vector<T> r((size_t)nc + nv, (T)0), last;
                 kind[k].resize(n);
                 for (int t = 0; t < n; ++t) {
-                    bool same = t > 0;                       // as the neighbour's, mostly
-                    for (size_t w = 0; w < r.size(); ++w) {
-                        same = same && r[w] == im[w * n + t];
-                        r[w] = im[w * n + t];
+                    int x, y;
+                    if (block(t, &x, &y)) fm[s][t] |= record(x, y, r.data(), 1);
+                    else r.assign(r.size(), (T)0);
+                    if (t > 0 && r == last) {                // the neighbour's, mostly
+                        kind[k][t] = kind[k][t - 1];
+                        continue;
                     }
-                    kind[k][t] = same ? kind[k][t - 1] : seen.emplace(r, (int)seen.size()).first->second;
+                    kind[k][t] = seen.emplace(r, (int)seen.size()).first->second;
+                    last = r;
                 }
                 nr = seen.size();
                 im.assign(r.size() * nr, (T)0);
                 for (const auto &q : seen)
                     for (size_t w = 0; w < r.size(); ++w) im[w * nr + q.second] = q.first[w];
+            } else {
+                im.assign((size_t)(nc + nv) * n, (T)0);
+                for (int t = 0; t < n; ++t) {
+                    int x, y;
+                    if (block(t, &x, &y)) fm[s][t] |= record(x, y, &im[t], n);
+                }
             }
             st.nrec[k] = (int)nr;
             table[s][k] = std::move(im);
