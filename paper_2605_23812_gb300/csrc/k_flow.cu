@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) k_correct(Grid g, double x0, double y0, d
     if (blockIdx.x == 0 && tid == 0) {
         double dv = g.dt * pt.red[m].val[RS_RMAX] / g.hxy;
         if (dv > ctl[m].max_div) ctl[m].max_div = dv;
-        if (!(dv <= div_tol)) ctl[m].status |= ENVAR_ST_DIVERGENCE;
+        if (!(dv <= div_tol)) atomicOr(&ctl[m].status, ENVAR_ST_DIVERGENCE);   // (other blocks set other bits)
         if (t > 0 && series) {
             double s[8];
             sample_sensors(g, x0, y0, usm, vsm, xm, s);

@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(256, 5) k_correct_mx(Grid g, MixConst K, MixSt
     if (blockIdx.x == 0 && tid == 0) {
         double dv = g.dt * pt.red[m].val[RS_RMAX] / g.hxy;
         if (dv > ctl[m].max_div) ctl[m].max_div = dv;
-        if (!(dv <= div_tol)) ctl[m].status |= ENVAR_ST_DIVERGENCE;
+        if (!(dv <= div_tol)) atomicOr(&ctl[m].status, ENVAR_ST_DIVERGENCE);   // (other blocks set other bits)
         if (t > 0 && series) {
             double sv[8];
             sample_sensors_mx(g, K, x0, y0, ush, usl, vsh, vsl, xh, xl, sv);
