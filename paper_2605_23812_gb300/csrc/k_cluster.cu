@@ -11,13 +11,15 @@
 // prolongation are register sums.  Consecutive block rows form a slab per thread block of the
 // cluster.  East / west neighbours come by shuffle, the others from a shared-memory plane that
 // holds every thread's border cells; slab borders are pushed into the neighbouring block's plane
-// with st.async, whose bytes complete a barrier there (one hop instead of a cluster barrier: 660
-// cycles with 1024 threads, measured).  The coarser levels are gathered in the cluster's first block
-// and run the same way on its first warps (stages 1, 2), with a named barrier between half-sweeps.
+// with st.async, whose bytes complete a barrier there: 690 cycles from store to use, 465 to 665 for a
+// barrier of the whole cluster (each measured by itself), but only the threads of a border wait for it.  The
+// coarser levels are gathered in the cluster's first block and run the same way on its first warps
+// (stages 1, 2), with a named barrier between half-sweeps.
 //
 // Red-black Gauss-Seidel does not depend on how cells are spread over threads, and every update
 // uses the operations of the tiled kernels in their order, so FP32 iterates equal theirs bit for bit;
-// dot products are df64 (or FP64) sums in another order.
+// dot products are df64 (or FP64) sums in another order, so a step length may round differently: runs of a
+// few steps had the same bits in every case compared, runs of 30 000 steps differ in the eighth digit of J.
 //
 // Every wait on a barrier in shared memory has an iteration limit.  A thread whose wait ran out sends
 // nothing more to other blocks and waits for nothing more, so the others' waits run out too; all blocks
@@ -284,8 +286,17 @@ __device__ __forceinline__ void ldg_row(const double *p, double (&v)[4])
 // Make the border cells of every block visible to its neighbours: into the stage's plane, and (stage
 // 0) into the neighbouring slabs' planes.  Two halo barriers per side, used in turn: a neighbour can
 // be at most one exchange ahead (its next push waits for this block's), so its bytes never meet the
-// barrier of the exchange before.  A halo row is read by the threads that push the opposite way, and a
-// neighbour waits for all of those pushes before it overwrites the row.
+// barrier of the exchange before.
+//
+// A halo row has one buffer, and a neighbour may push the next one while this block still reads it: it waited
+// for this block's push of the same exchange, which comes before the read.  The same holds for a block's own
+// border cells in its plane, which it stores without waiting for the last read of them.  Both rely on this, and
+// every use has to keep it:
+//   - two exchanges of a plane with nothing between them but a half-sweep differ only in the colour that the
+//     half-sweep updates, and it reads the other one: what it reads is overwritten with the same values;
+//   - a read of both colours (residual, q = A p) is followed by an exchange of another level's plane, by the
+//     gather or by a sum over the cluster before the plane is written again, and none of these gets
+//     past a block that has not finished the read.
 template <class T, int b, int S, bool MULTI>
 __device__ __forceinline__ void exchange(Ctx<T, S> &c, int k, const T (&e)[b][b])
 {
@@ -1030,7 +1041,7 @@ __device__ __forceinline__ double outer_res(const ClusterArgs &a, const SolveArg
 // Fluid sum of x (its high words), in the order of k_outer_residual_mx and res_finish_member: warps of
 // 64 columns x 4 rows, blocks of eight of them, then the blocks' partials by one warp.  The mean it
 // gives enters the pressure and the next guess, and cancels almost to zero, so its bits depend on the
-// order; mixed handles take the same bits on either solve path.
+// order; mixed handles sum in the same order on either solve path.
 template <bool MULTI>
 __device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<float, 0> &c, long long off, int turn, bool *failed)
 {
@@ -1096,8 +1107,8 @@ __device__ double fluid_sum_mx(const ClusterArgs &a, const SolveArgs &sa, Ctx<fl
 // iterate and right-hand side (32 values) with one level's conductances (16) in 96 registers.
 // FP64 2 x 2 blocks: 152 registers without spills up to 192 threads, with which two blocks still share an SM;
 // beyond, 128 (512 threads), for the same reason.  (At 80 registers and 768 threads 400 bytes per thread spilled: 128 x 64,
-// one member at a time: 50.5 ms, now 42.5 ms; 176 x 80, 17 members: 10.4 ms, with 152 registers and one block per
-// SM 13.7 ms, with 128 registers 9.4 ms.)
+// one member at a time: 51.7 ms, now 43.3 ms; 176 x 80, 17 members: 10.4 ms, with 152 registers and one block per
+// SM 13.7 ms, with 128 registers 10.0 ms.)
 constexpr int CL_FEW_THREADS = 192, CL_FEW_BOUND = 384;
 // Mixed 4 x 4 blocks up to 512 threads: 128 registers where an SM holds one block anyway (more than 320 threads,
 // or 112 KB; 96 registers spill 460 bytes per thread): 256 x 128, 33 members 7.31 -> 6.56 ms, 5 members 2.96 -> 2.70 ms.
@@ -1848,7 +1859,7 @@ ClusterPlan *cluster_plan(const ClusterHostLevel *hl, int nlev, int ncoarse, boo
         // The smallest cluster that holds the grid, rounded up to the largest size of which as many are
         // resident (clusters at 180 KB per block, measured: 2: 76, 3 and 4: 36, 5: 28, 6: 23, 7 to 9: 15,
         // 10: 13, 12: 8, 14 and 16: 7): more SMs per member that no other member could use (256 x 128, 33
-        // members: 3 blocks 8.1 ms, 4 blocks 7.5 ms, 5 blocks 7.9 ms).
+        // members: 3 blocks 7.8 ms, 4 blocks 7.4 ms, 5 blocks 7.9 ms).
         for (int C : {1, 2, 4, 3, 5, 6, 9, 8, 7, 10, 12, 14, 16}) cand.push_back({4, C});
     } else if (la == 0) {
         // FP64 issues one warp instruction per scheduler in 64 cycles (0.49 FMA per clock and warp, 1.67 per
