@@ -19,10 +19,8 @@ Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|referen
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
-import re
 import statistics
 import subprocess
 import sys
@@ -196,23 +194,6 @@ def reference_arm(args, dist):
 
 
 # ------------------------------------------------------------------------------------------------
-def kernel_traffic(summary: str, sweeps: int):
-    """DRAM bytes per launch from a committed ncu summary under profiles/, if the kernel's source
-    file is unchanged since the capture (its 'source' line holds the file and its sha256 prefix)
-    and the captured instantiation has the sweep count the run uses (its 'sweeps' line)."""
-    path = os.path.join(ROOT, "profiles", summary)
-    try:
-        text = open(path).read()
-        if int(re.search(r"^sweeps:\s*(\d+)", text, re.M).group(1)) != sweeps:
-            return None
-        traffic = float(re.search(r"^traffic_bytes_per_launch:\s*([0-9.eE+]+)", text, re.M).group(1))
-        src, sha = re.search(r"^source:\s*(\S+)\s+sha256\[:16\]\s*=\s*([0-9a-f]{16})", text, re.M).groups()
-        cur = hashlib.sha256(open(os.path.join(ROOT, src), "rb").read()).hexdigest()[:16]
-    except (OSError, AttributeError, ValueError):
-        return None
-    return traffic if cur == sha else None
-
-
 def regime(series, dt):
     """Flow regime of the unperturbed member over the cost window from its sensor series
     [n_window][8] (u, v at x = 1/5 .. 4/5, y = 0; Sec. 4.1): rms of the fluctuation of each channel,
@@ -317,13 +298,18 @@ def gb300_arm(args, dist):
 
     out = None
     if dist.rank == 0:
-        # roofline of the dominant kernel (level-0 multigrid prolongation + post-smoothing + dot), timed
-        # live on the handle's stream with a cold L2; algorithmic bytes: f, input guess, output (4 B each) and the
-        # coarse correction (1 B per fine cell) per cell and member, plus the open-face bits (1 B per
-        # cell, shared by the members)
+        # The pressure solve (k_cluster, about three quarters of a step) keeps its vectors on chip and is bound by
+        # latency: it has no bandwidth to hold against the memory's.  The roofline line is the largest
+        # memory-bound kernel that the iteration launches, the projection correction in the cost window, timed
+        # live on the handle's stream with a cold L2.  Algorithmic bytes per fluid cell: u*, v* (16), x (8), u, v
+        # (16), p read and written (8), six Welford planes read and written (48); members but the first the Welford of
+        # u - u_0 (32); member 0's velocity (16), shared.
         with torch.cuda.stream(stream):
-            ms = ens.time_kernel(2, 20)
-        algo_bytes = 13.0 * NX * NY * M + 1.0 * NX * NY
+            ms = ens.time_kernel(6, 20)
+        x = cfg.x0 + (np.arange(NX) + 0.5) * (cfg.x1 - cfg.x0) / NX
+        y = cfg.y0 + (np.arange(NY) + 0.5) * (cfg.y1 - cfg.y0) / NY
+        fluid = int(((y[:, None] > 0) | ((x > 0) & (x < 1))[None, :]).sum())
+        algo_bytes = fluid * (96.0 * M + 32.0 * (M - 1) + 16.0)
         achieved = algo_bytes / (ms * 1e-3) / 1e9
         peaks = {}
         try:
@@ -331,15 +317,13 @@ def gb300_arm(args, dist):
         except (OSError, ValueError):
             pass
         peak = peaks.get("hbm_gbs", 6800.0)
-        traffic = kernel_traffic("k_smoothw_l0_post_512x256x33.md", solver["nu"])
-        roof = {"kernel": f"k_smoothw<float,{solver['nu']},12,0> (level-0 prolongation + post-smoothing + r.z)",
+        roof = {"kernel": "k_correct_mx (projection correction with the Welford updates)",
                 "bound": "hbm",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
-                "traffic": traffic, "launch_ms": ms,
-                "achieved_dram": (traffic / (ms * 1e-3) / 1e9) if traffic else None,
-                "achieved_note": "achieved = algorithmic bytes / launch time; achieved_dram = ncu DRAM bytes / "
-                                 "launch time",
+                "traffic": None, "launch_ms": ms,
+                "achieved_note": "achieved = algorithmic bytes of the fluid cells / launch time; the pressure solve "
+                                 "(k_cluster) is bound by latency and has no roofline line",
                 "timing": "cold L2 (256 MB write before each launch), mean of 20 launches"}
         # the plain one-member-at-a-time FP64 GPU path: one member of the iteration, every one of its
         # 30 000 steps timed (all 33 members run the same horizon from the same initial state)
