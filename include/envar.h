@@ -291,7 +291,7 @@ int envar_time_kernel(envar_handle h, int which, int reps, double *ms_per_launch
  * member slot 0 (r_dev, z_dev: [ny][nx] float64, device; solid cells of r must be zero).  M is
  * one symmetric V-cycle (red-black Gauss-Seidel, cell-sum restriction, piecewise-constant
  * prolongation) and must be symmetric positive definite on mean-zero fields.  Overwrites the
- * solver's work vectors of every member slot. */
+ * solver's work vectors of every member slot.  ENVAR_ESTATE: a wait inside the V-cycle ran out, z is not valid. */
 int envar_apply_preconditioner(envar_handle h, const double *r_dev, double *z_dev);
 
 /* Diagnostics of one handle, for tests (a batch that holds the handle keeps what it has captured).

@@ -1997,7 +1997,13 @@ extern "C" int envar_apply_preconditioner(envar_handle h, const double *r_dev, d
     CK(cudaMemsetAsync(h->pb.lev_f[1], 0, tsz * (size_t)h->lev[1].S * h->Mall, h->st));
     CK(cudaMemsetAsync(h->pb.z, 0, tsz * (size_t)h->g.S, h->st));
     CK(cudaMemsetAsync(h->pb.lev_t[0], 0, tsz * (size_t)h->lev[0].S, h->st));
+    int status = 0;
+    CK(cudaMemcpyAsync(&status, &h->d_ctl[0].status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));
+    if (status) {
+        set_err(h, "envar_apply_preconditioner: status 0x%x (a wait between the blocks of the V-cycle ran out)", status);
+        return ENVAR_ESTATE;
+    }
     CK(cudaGetLastError());
     return ENVAR_OK;
 }

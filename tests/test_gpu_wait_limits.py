@@ -45,3 +45,17 @@ def test_a_wait_that_runs_out_is_reported(nx, ny, precision, conditional):
     assert (status == 0).all() and (status0 == 0).all()
     for a, b in zip(state, state0):
         assert np.array_equal(a, b)
+
+
+def test_a_preconditioner_application_that_ran_out_is_refused():
+    nx, ny = 1024, 512
+    ens = pkg.Ensemble(pkg.default_config(nx, ny, n_members=1, n_steps=2, n_window=1, precision=pkg.MIXED))
+    r = np.random.default_rng(0).standard_normal((ny, nx))
+    r[:ny // 2] = 0.0                                        # the channel's cells alone: zero in solid cells
+    z = ens.apply_preconditioner(r).cpu().numpy()
+    ens.set_diagnostic(WAIT_LIMIT, 0)
+    with pytest.raises(pkg.EnvarError):
+        ens.apply_preconditioner(r)
+    ens.set_diagnostic(WAIT_LIMIT, -1)
+    assert np.array_equal(z, ens.apply_preconditioner(r).cpu().numpy())
+    ens.close()
